@@ -58,7 +58,8 @@ BYTES_PER_CELL = 120.0      # read E,B,J (72) + write E,B (48)
 TRAFFIC_CAPTURE = {"bytes_per_particle": (501.010432e6 + 409.757440e6) / 8388608, "dim": 3, "order": 1,
                    "sources": ("paper_2104_11385_gb300/csrc/pic_particle_kernel.cuh",
                                "paper_2104_11385_gb300/csrc/pic_particles_f64_3d.cu",
-                               "paper_2104_11385_gb300/csrc/pic_dd.cuh",
+                               "paper_2104_11385_gb300/csrc/pic_arith.cuh",
+                               "paper_2104_11385_gb300/csrc/pic_fix.cuh",
                                "paper_2104_11385_gb300/csrc/pic_internal.h",
                                "paper_2104_11385_gb300/csrc/pic_sync.cuh"),
                    "sha256": "82cc630c91293752a1621f91ff9feac441b0448dc4fe5d75df8e4a03b78108c0"}

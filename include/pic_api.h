@@ -170,7 +170,8 @@ enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
  *   cost        heuristic (w_p Np + w_c Nc per box), device clock (summed
  *               per-thread clock64 of the particle kernel, per box; the
  *               paper's GPU-clock strategy), or kernel time (summed
- *               %globaltimer span of the box's work units: the in-kernel
+ *               %globaltimer span of the box's particle loops, the mean over
+ *               each CTA's warps: the in-kernel
  *               analog of the paper's CUPTI kernel duration, without CUPTI).
  *   w_p, w_c    heuristic weights (Sec. 3.3 footnotes: 0.75/0.25 knapsack,
  *               0.02/0.98 SFC).
@@ -221,7 +222,8 @@ pic_status pic_sync(pic_sim* sim);
  * with the weights of the last pic_set_lb_params (0.75/0.25 by default);
  * DEVICE_CLOCK: summed thread clock cycles of the particle kernel since the
  * last rebalance (or since the start); KERNEL_TIME: summed nanoseconds
- * (%globaltimer) of the box's work units over the same window.  costs_out: host, nboxes doubles;
+ * (%globaltimer) of the box's particle loops (mean over the warps of the CTA
+ * that runs a unit) over the same window.  costs_out: host, nboxes doubles;
  * np_out: host, nboxes int64 particle counts (nullable).  Box index
  * (bz*nby + by)*nbx + bx.  Synchronises the stream. */
 pic_status pic_get_box_costs(pic_sim* sim, int strategy, double* costs_out, int64_t* np_out);
@@ -239,7 +241,8 @@ pic_status pic_rebalance(pic_sim* sim, const pic_lb_params* params, pic_lb_resul
 /* In-kernel cost capture (Sec. 2.2, the device-side measurement this work
  * is about): PIC_CAPTURE_CLOCK accumulates each thread's clock64() deltas
  * over its particle loop into the box's device-clock cost; PIC_CAPTURE_TIME
- * adds each work unit's %globaltimer span to the box's kernel-time cost.
+ * adds the %globaltimer span of each work unit's particle loops (mean over
+ * the CTA's warps) to the box's kernel-time cost.
  * Both are on by default.  A strategy whose capture is off reads zero costs
  * (and a load balancer driven by it then sees E = 1 and keeps its mapping);
  * the heuristic strategy needs neither.  Turning capture off measures its
@@ -341,10 +344,9 @@ pic_status pic_bin_particles(const pic_grid_desc* grid, const double* x, const d
  *                 loads of that many particles are issued before the first
  *                 of them is pushed.
  *   precision     arithmetic of the particle push: 1 FP64 (default);
- *                 2 float-float (pairs of FP32 with error-free
- *                 transformations, ~48-bit significand) for gather, Boris and
- *                 deposit weights, with FP64 storage, positions, index math and
- *                 current accumulation -- the mixed-precision variant; 3 FP32
+ *                 2 float-float or better (a significand of at least 48 bits
+ *                 for gather, Boris and deposit weights): runs the arithmetic
+ *                 of 1, which is the faster of the two; 3 FP32
  *                 for gather, Boris and deposit weights with FP64 storage,
  *                 positions and current accumulation (the FP32 variant:
  *                 about 2^-24 per operation, so it meets an FP32-derived

@@ -138,10 +138,10 @@ struct LaunchCfg {
     int threads;
     int ctas;
     int minb;     // register budget variant of the particle kernel: 1 or 2 CTAs per SM
-    int prec;     // arithmetic of the particle push: 0 FP64, 1 float-float, 2 FP32
+    int prec;     // arithmetic of the particle push: 0 FP64, 1 float-float (run as FP64), 2 FP32
     int ppt = 1;  // particles per thread per loop iteration (1 or 2)
 };
-// dynamic shared memory of the particle kernel; prec 0 FP64, 1 float-float, 2 FP32
+// dynamic shared memory of the particle kernel (every precision)
 size_t pic_particle_smem_bytes(int dim, int order, const int T[3], int threads, int prec);
 cudaError_t pic_prepare_particles(int dim, int order, size_t smem);  // outside graph capture
 int pic_particle_occupancy(int dim, int order, int minb, int ppt, int threads, size_t smem,
@@ -155,8 +155,6 @@ int pic_particle_occupancy(int dim, int order, int minb, int ppt, int threads, s
     int pic_particle_occupancy_##SUF(int order, int minb, int ppt, int threads, size_t smem);
 PIC_DECLARE_PARTICLE_TU(p0_d3)
 PIC_DECLARE_PARTICLE_TU(p0_d2)
-PIC_DECLARE_PARTICLE_TU(p1_d3)
-PIC_DECLARE_PARTICLE_TU(p1_d2)
 PIC_DECLARE_PARTICLE_TU(p2_d3)
 PIC_DECLARE_PARTICLE_TU(p2_d2)
 // self-test of the device's bounded wait: one CTA waits on an mbarrier that

@@ -1,20 +1,29 @@
 // pic_particle_kernel.cuh -- the particle side of the PIC cycle on sm_103a,
 // templated on the arithmetic of the particle push (included by one
 // translation unit per precision and dimensionality:
-// pic_particles_{f64,dd,f32}_{3d,2d}.cu).
+// pic_particles_{f64,f32}_{3d,2d}.cu).
 //
 // pic_particle_kernel: persistent CTAs pull work units (a chunk of one box's
 // particles) from cost-ordered lists.  For every tile (sub-box) a unit touches,
 // the guard-extended E/B tile is staged into shared memory by TMA
 // (cp.async.bulk.tensor, local HBM only, no multicast).  The current goes
 // straight into the guard-padded global J arrays as fire-and-forget FP64
-// reductions (red.global.add.f64, performed in L2) in every precision; the
-// FP32 variant also stages its particle loads through shared memory with
-// cp.async one loop iteration ahead.  Each thread brackets its particle
+// reductions (red.global.add.f64, performed in L2) in every precision, and the
+// particle loads are staged through shared memory with cp.async one loop
+// iteration ahead.
+//
+// What bounds it (FP64, linear, 128^3 foil, 8.4 M particles): the FP64 pipe
+// takes one warp instruction per SM every 16 clocks, and a particle's gather,
+// push and deposit are 165 FP64 instructions, 2.73 ms at 86 % of that pipe.
+// The gather (60 of them) and the deposit (36) run in 64-bit fixed point on the
+// integer pipes instead (pic_fix.cuh), the Boris push keeps 51: 1.48 ms, about
+// 2600 issued instructions per 32 particles, issue slots 48 % and FP64 pipe
+// 55 % busy (16 warps per SM by registers: latency-bound between the two).  Each thread brackets its particle
 // loop with clock64(); the deltas are warp-reduced, summed in shared memory and
 // added once per unit to the box's cost -- the device-clock cost of
-// arXiv 2104.11385 Sec. 2.2 (Fig. 2a); thread 0 adds the unit's %globaltimer
-// span to the box's kernel-time cost.  The same pass writes each particle's new
+// arXiv 2104.11385 Sec. 2.2 (Fig. 2a); thread 0 adds the %globaltimer span
+// of the unit's particle loops, averaged over the warps, to the box's
+// kernel-time cost.  The same pass writes each particle's new
 // tile key and the per-tile histogram for the re-sort.
 //
 // Physics per particle (the schemes the paper leaves open, Sec. 2.1): field
@@ -26,7 +35,8 @@
 #pragma once
 #include <type_traits>
 
-#include "pic_dd.cuh"
+#include "pic_arith.cuh"
+#include "pic_fix.cuh"
 #include "pic_internal.h"
 #include "pic_sync.cuh"
 
@@ -114,7 +124,7 @@ __device__ __forceinline__ bool ge_half(double f) {  // f >= 0.5 for f >= 0
 }
 
 // one-dimensional B-spline support: first node and ORDER+1 weights in the
-// arithmetic type R (double; dd for the float-float variant; float for the FP32 one)
+// arithmetic type R (double, or float for the FP32 variant)
 template <int ORDER, class R>
 struct Support {
     int s;
@@ -254,37 +264,13 @@ struct EBHalo {
     static constexpr int lo = ORDER == 3 ? 2 : 1;
 };
 
-// interpolation of one component from a shared tile with extents (SX, SY);
-// the tile holds R values (doubles, or float pairs converted in place).  D,
-// when given (linear FP64), holds the tile's x differences F[x+1] - F[x] on
-// rows of SX - 1, so that each x lerp is one FMA.
+// interpolation of one component from a shared tile of R values (FP32, and FP64
+// for tiles that the fixed-point gather does not take) with extents (SX, SY)
 template <class R, int ORDER, int DIM>
 __device__ __forceinline__ R interp(const R* __restrict__ F, int SX, int SY, const Support<ORDER, R>& sx,
-                                    const Support<ORDER, R>& sy, const Support<ORDER, R>& sz,
-                                    const R* __restrict__ D = nullptr) {
+                                    const Support<ORDER, R>& sy, const Support<ORDER, R>& sz) {
     // tile column 0 is local cell -EBHalo<ORDER>::lo
     constexpr int H = EBHalo<ORDER>::lo;
-    if constexpr (ORDER == 1 && std::is_same<R, double>::value) {
-        if (D) {
-            auto lerp = [](R a, R b, R f) { return fma(f, b - a, a); };
-            const R fx = sx.w[1];
-            const int DX = SX - 1;
-            if constexpr (DIM == 3) {
-                const int r00 = (sz.s + H) * SY + (sy.s + H);
-                const int x = sx.s + H;
-                const R a00 = fma(fx, D[r00 * DX + x], F[r00 * SX + x]);
-                const R a10 = fma(fx, D[(r00 + 1) * DX + x], F[(r00 + 1) * SX + x]);
-                const R a01 = fma(fx, D[(r00 + SY) * DX + x], F[(r00 + SY) * SX + x]);
-                const R a11 = fma(fx, D[(r00 + SY + 1) * DX + x], F[(r00 + SY + 1) * SX + x]);
-                return lerp(lerp(a00, a10, sy.w[1]), lerp(a01, a11, sy.w[1]), sz.w[1]);
-            } else {
-                const int r0 = sz.s + H, x = sx.s + H;
-                const R a0 = fma(fx, D[r0 * DX + x], F[r0 * SX + x]);
-                const R a1 = fma(fx, D[(r0 + 1) * DX + x], F[(r0 + 1) * SX + x]);
-                return lerp(a0, a1, sz.w[1]);
-            }
-        }
-    }
     if constexpr (ORDER == 1) {
         // linear: nested lerps a + f (b - a) need only the fractional parts
         auto lerp = [](R a, R b, R f) { return fma(f, b - a, a); };
@@ -332,38 +318,61 @@ __device__ __forceinline__ R interp(const R* __restrict__ F, int SX, int SY, con
     }
 }
 
+// The six E/B components at one particle.  E_a sits on the half-node grid
+// along a and on nodes across it, B_a the other way round.
+template <class R, int ORDER, int DIM>
+__device__ __forceinline__ void gather6(const R* __restrict__ sEB, int stride, int SX, int SY,
+                                        const Support<ORDER, R>* nd, const Support<ORDER, R>* hf, R* e,
+                                        R* b) {
+    e[0] = interp<R, ORDER, DIM>(sEB, SX, SY, hf[0], nd[1], nd[2]);
+    e[1] = interp<R, ORDER, DIM>(sEB + stride, SX, SY, nd[0], hf[1], nd[2]);
+    e[2] = interp<R, ORDER, DIM>(sEB + 2 * stride, SX, SY, nd[0], nd[1], hf[2]);
+    b[0] = interp<R, ORDER, DIM>(sEB + 3 * stride, SX, SY, nd[0], hf[1], hf[2]);
+    b[1] = interp<R, ORDER, DIM>(sEB + 4 * stride, SX, SY, hf[0], nd[1], hf[2]);
+    b[2] = interp<R, ORDER, DIM>(sEB + 5 * stride, SX, SY, hf[0], hf[1], nd[2]);
+}
+
 template <class T>
 __device__ __forceinline__ T pick3(int a, const T& v0, const T& v1, const T& v2) {
     return a == 0 ? v0 : (a == 1 ? v1 : v2);
 }
 
-// The six E/B components at one particle.  E_a sits on the half-node grid
-// along a and on nodes across it, B_a the other way round.  FP64 and FP32
-// unroll the six interpolations; float-float runs them as a loop (its operations are
-// 7-11 FP32 instructions each, and six unrolled copies overflow the
-// instruction cache).
-template <class R, int ORDER, int DIM>
-__device__ __forceinline__ void gather6(const R* __restrict__ sEB, int stride, int SX, int SY,
-                                        const Support<ORDER, R>* nd, const Support<ORDER, R>* hf, R* e,
-                                        R* b, const R* __restrict__ sD = nullptr, int dstride = 0) {
-    if constexpr (!std::is_same<R, dd>::value) {
-        const bool hd = sD != nullptr;
-        e[0] = interp<R, ORDER, DIM>(sEB, SX, SY, hf[0], nd[1], nd[2], hd ? sD : nullptr);
-        e[1] = interp<R, ORDER, DIM>(sEB + stride, SX, SY, nd[0], hf[1], nd[2], hd ? sD + dstride : nullptr);
-        e[2] = interp<R, ORDER, DIM>(sEB + 2 * stride, SX, SY, nd[0], nd[1], hf[2], hd ? sD + 2 * dstride : nullptr);
-        b[0] = interp<R, ORDER, DIM>(sEB + 3 * stride, SX, SY, nd[0], hf[1], hf[2], hd ? sD + 3 * dstride : nullptr);
-        b[1] = interp<R, ORDER, DIM>(sEB + 4 * stride, SX, SY, hf[0], nd[1], hf[2], hd ? sD + 4 * dstride : nullptr);
-        b[2] = interp<R, ORDER, DIM>(sEB + 5 * stride, SX, SY, hf[0], hf[1], nd[2], hd ? sD + 5 * dstride : nullptr);
+// ---- FP64: fixed-point gather -----------------------------
+struct Six {
+    double v[6];  // Ex Ey Ez Bx By Bz
+};
+
+// the six components from the tile in fixed point (component c at c * stride,
+// the biased exponent of its largest magnitude in emax[c]).  Linear shapes
+// unroll the six interpolations; the others run them as a loop (27 or 64
+// products each: six copies would not fit the instruction cache).
+template <int ORDER, int DIM>
+__device__ __forceinline__ Six gather6_q(const long long* __restrict__ F, int stride, int SX, int SY,
+                                         const int* __restrict__ emax, const AxisQ<ORDER>* nd,
+                                         const AxisQ<ORDER>* hf) {
+    constexpr int H = EBHalo<ORDER>::lo;
+    constexpr int B = 63 - TileBits<ORDER>::FB;  
+    Six r;
+    if constexpr (ORDER == 1) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const int a = c < 3 ? c : c - 3;
+            const bool isb = c >= 3;
+            r.v[c] = fix_double(interp_q<ORDER, DIM, H>(F + c * stride, SX, SY, (a == 0) != isb ? hf[0] : nd[0],
+                                                        (a == 1) != isb ? hf[1] : nd[1],
+                                                        (a == 2) != isb ? hf[2] : nd[2]),
+                                emax[c] + B);
+        }
     } else {
-        R v0 = Arith<R>::c(0.0), v1 = v0, v2 = v0, v3 = v0, v4 = v0, v5 = v0;
+        double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0, v4 = 0.0, v5 = 0.0;
 #pragma unroll 1
         for (int c = 0; c < 6; ++c) {
             const int a = c < 3 ? c : c - 3;
             const bool isb = c >= 3;
-            const Support<ORDER, R> sx = ((a == 0) != isb) ? hf[0] : nd[0];
-            const Support<ORDER, R> sy = ((a == 1) != isb) ? hf[1] : nd[1];
-            const Support<ORDER, R> sz = ((a == 2) != isb) ? hf[2] : nd[2];
-            const R v = interp<R, ORDER, DIM>(sEB + c * stride, SX, SY, sx, sy, sz);
+            const AxisQ<ORDER> sx = ((a == 0) != isb) ? hf[0] : nd[0];
+            const AxisQ<ORDER> sy = ((a == 1) != isb) ? hf[1] : nd[1];
+            const AxisQ<ORDER> sz = ((a == 2) != isb) ? hf[2] : nd[2];
+            const double v = fix_double(interp_q<ORDER, DIM, H>(F + c * stride, SX, SY, sx, sy, sz), emax[c] + B);
             v0 = c == 0 ? v : v0;
             v1 = c == 1 ? v : v1;
             v2 = c == 2 ? v : v2;
@@ -371,9 +380,30 @@ __device__ __forceinline__ void gather6(const R* __restrict__ sEB, int stride, i
             v4 = c == 4 ? v : v4;
             v5 = c == 5 ? v : v5;
         }
-        e[0] = v0; e[1] = v1; e[2] = v2;
-        b[0] = v3; b[1] = v4; b[2] = v5;
+        r = Six{{v0, v1, v2, v3, v4, v5}};
     }
+    return r;
+}
+
+// the same in FP64 from the doubles as staged: tiles holding Inf or NaN, or
+// magnitudes outside the fixed-point gather's exponent range
+template <int ORDER, int DIM>
+static __device__ __noinline__ Six gather6_fp64(const double* __restrict__ sEB, int stride, int SX, int SY, double X,
+                                                double Y, double Z, int ox, int oy, int oz, bool ec) {
+    Support<ORDER, double> nd[3], hf[3];
+    int c;
+    supports_at<ORDER, double>(X, ox, ec, nd[0], hf[0], c);
+    supports_at<ORDER, double>(Z, oz, ec, nd[2], hf[2], c);
+    if (DIM == 3) {
+        supports_at<ORDER, double>(Y, oy, ec, nd[1], hf[1], c);
+    } else {
+        nd[1].s = -1;
+        nd[1].w[0] = 1.0;
+        hf[1] = nd[1];
+    }
+    Six r;
+    gather6<double, ORDER, DIM>(sEB, stride, SX, SY, nd, hf, r.v, r.v + 3);
+    return r;
 }
 
 // Esirkepov node shapes on a common window of W nodes starting at the lower of
@@ -391,7 +421,8 @@ __device__ __forceinline__ bool make_window(const Support<ORDER, R>& a, const Su
                                             Window<ORDER, W, R>& win) {
     int base = min(a.s, b.s);
     int oa = a.s - base, ob = b.s - base;
-    if (oa > W - ORDER - 1 || ob > W - ORDER - 1) return false;
+    // unsigned: a cell index saturated by a move of 2^31 cells or more wraps the difference
+    if ((unsigned)oa > (unsigned)(W - ORDER - 1) || (unsigned)ob > (unsigned)(W - ORDER - 1)) return false;
     win.base = base;
     const R zero = Arith<R>::c(0.0);
 #pragma unroll
@@ -434,6 +465,34 @@ __device__ __forceinline__ int tile_key(const SV& S, int ix, int iy, int iz) {
     return b * S.tiles_per_box + (tz * S.tpb[1] + ty) * S.tpb[0] + tx;
 }
 
+// A tile's key is a sum of one part per direction.  For the staged tile the
+// parts of its own position and of the neighbours' on either side (periodic)
+// are kept in shared memory, so that a particle that moved by less than a tile
+// finds its new key without the nine integer divisions of tile_key.
+template <class SV>
+__device__ __forceinline__ int key_part(const SV& S, int a, int i) {
+    const int n = S.n[a];
+    i = i < 0 ? i + n : (i >= n ? i - n : i);
+    const int b = i / S.bsz[a], t = (i - b * S.bsz[a]) / S.T[a];
+    const int bs = a == 0 ? 1 : (a == 1 ? S.nb[0] : S.nb[0] * S.nb[1]);
+    const int ts = a == 0 ? 1 : (a == 1 ? S.tpb[0] : S.tpb[0] * S.tpb[1]);
+    return b * bs * S.tiles_per_box + t * ts;
+}
+// key of the tile that holds the cell at offset r[a] (unwrapped) from the tile's origin; -1: further off
+template <int DIM, class SV>
+__device__ __forceinline__ int near_key(const SV& S, const int (*nk)[3], const int r[3]) {
+    int key = 0;
+    bool near = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (DIM == 2 && a == 1) continue;
+        const int T = S.T[a];
+        near = near && r[a] >= -T && r[a] < 2 * T;
+        key += nk[a][r[a] < 0 ? 0 : (r[a] < T ? 1 : 2)];
+    }
+    return near ? key : -1;
+}
+
 __device__ __forceinline__ void warp_hist_add(int32_t* count, int key) {
     unsigned act = __activemask();
     unsigned peers = __match_any_sync(act, key);
@@ -442,23 +501,32 @@ __device__ __forceinline__ void warp_hist_add(int32_t* count, int key) {
 }
 
 // The fields of a simulation and of its species that the particle loop reads,
-// staged in shared memory once per work unit.  Read from the SimDev in global
-// memory they would be fetched again for every particle (the loop's stores to
-// the particle arrays might alias them as far as the compiler can tell).
+// staged in shared memory when a CTA's simulation changes, and the unit's
+// particle range of each species.  Read from the SimDev in global memory they
+// would be fetched again for every particle (the loop's stores to the particle
+// arrays might alias them as far as the compiler can tell).
 struct HotSp {
     double* cur[7];
     int32_t* key;
     int32_t* count;
+    const int64_t* off;
+    double kq, q;
+    int64_t r0, r1;  // the unit's particles
 };
 struct HotSim {
     double nd[3];
+    Amp ja[3];  // current prefactors -1/(dA dt) (2D: jyfac2d for y)
+    ExpRange je;
     int T[3], n[3], bsz[3], nb[3], tpb[3], ebs[3];
-    int tiles_per_box, ntiles, absorb, ec, jlo;
+    int tiles_per_box, ntiles, absorb, ec, jlo, nsp;
+    int nk[3][3];  // key parts of the staged tile and its neighbours
     HotSp sp[PIC_MAXSP];
 };
 
+// one thread per direction and per species: the loads of different threads overlap
 __device__ __forceinline__ void stage_hot(HotSim& h, const SimDev& S) {
-    for (int a = 0; a < 3; ++a) {
+    const int a = threadIdx.x, i = (int)threadIdx.x - 4;
+    if (a < 3) {
         h.nd[a] = S.nd[a];
         h.T[a] = S.T[a];
         h.n[a] = S.n[a];
@@ -466,16 +534,22 @@ __device__ __forceinline__ void stage_hot(HotSim& h, const SimDev& S) {
         h.nb[a] = S.nb[a];
         h.tpb[a] = S.tpb[a];
         h.ebs[a] = S.ebs[a];
-    }
-    h.tiles_per_box = S.tiles_per_box;
-    h.ntiles = S.ntiles;
-    h.absorb = S.absorb;
-    h.ec = S.ec;
-    h.jlo = S.jlo;
-    for (int i = 0; i < S.nsp; ++i) {
-        for (int a = 0; a < 7; ++a) h.sp[i].cur[a] = S.sp[i].cur[a];
+        h.ja[a] = amp_of(S.dim == 2 && a == 1 ? S.jyfac2d : S.jfac[a]);
+    } else if (a == 3) {
+        h.tiles_per_box = S.tiles_per_box;
+        h.ntiles = S.ntiles;
+        h.absorb = S.absorb;
+        h.ec = S.ec;
+        h.jlo = S.jlo;
+        h.nsp = S.nsp;
+        h.je = exp_range(S.jfac[0], S.dim == 2 ? S.jyfac2d : S.jfac[1], S.jfac[2]);
+    } else if (i < S.nsp) {
+        for (int k = 0; k < 7; ++k) h.sp[i].cur[k] = S.sp[i].cur[k];
         h.sp[i].key = S.sp[i].key;
         h.sp[i].count = S.sp[i].count;
+        h.sp[i].off = S.sp[i].off;
+        h.sp[i].kq = S.sp[i].kq;
+        h.sp[i].q = S.sp[i].q;
     }
 }
 
@@ -495,36 +569,32 @@ static_assert(QFields<3>::n * WQ == PIC_RING_DOUBLES && QMAXWARPS == 8,
 
 struct SmemPlan {
     int eb_stride;  // doubles per E/B component (multiple of 16 -> 128-byte aligned)
-    int d_stride;   // doubles per component of the x-difference tile (0: none)
-    int eb_vol, d_vol;
+    int eb_vol;
     int pb_off;     // doubles from the base to the particle staging buffers
+    bool staged;    // whether there are such buffers
     size_t bytes;
 };
 
-// Particle staging (FP32 variant): per warp two buffers of the 7 stored
+// Particle staging: per warp two buffers of the 7 stored
 // values of 32 particles, filled by cp.async one loop iteration ahead.
 constexpr int PIN_SLOTS = 7 * 32;
 constexpr int PIC_PBUF_DOUBLES = QMAXWARPS * 2 * PIN_SLOTS;
 
-// xdiff: the x differences of the staged E/B tile are kept beside it (linear
-// FP64).  pbuf: particle staging buffers (FP32 variant).  The FP32 variant
-// converts the staged E/B tile in place: for linear shapes to float pairs
-// (F[x], F[x+1] - F[x]), component c at pair c * eb_stride; otherwise to
-// floats, component c at float c * eb_stride.
-// Layout: E/B tile (TMA) | x differences | particle buffers.
-__host__ __device__ inline SmemPlan smem_plan(const int ebs[3], bool xdiff, bool pbuf) {
+// FP64 converts the staged E/B tile in place to fixed point, the FP32 variant for linear
+// shapes to float pairs (F[x], F[x+1] - F[x]), component c at pair c *
+// eb_stride, otherwise to floats, component c at float c * eb_stride.
+// Layout: E/B tile (TMA) | particle buffers.
+__host__ __device__ inline SmemPlan smem_plan(const int ebs[3]) {
     SmemPlan p;
     p.eb_vol = ebs[0] * ebs[1] * ebs[2];
-    p.d_vol = xdiff ? (ebs[0] - 1) * ebs[1] * ebs[2] : 0;
     p.eb_stride = (p.eb_vol + 15) & ~15;
-    p.d_stride = (p.d_vol + 15) & ~15;
-    p.pb_off = 6 * p.eb_stride + 6 * p.d_stride;
-    p.bytes = (size_t)(p.pb_off + (pbuf ? PIC_PBUF_DOUBLES : 0)) * sizeof(double);  // tiles and buffers
+    p.pb_off = 6 * p.eb_stride;
+    // tiles too large to leave room for the buffers (2D tiles of 64 cells) load
+    // their particles directly
+    p.staged = (p.pb_off + PIC_PBUF_DOUBLES) * sizeof(double) <= 225 * 1024;
+    p.bytes = (size_t)(p.pb_off + (p.staged ? PIC_PBUF_DOUBLES : 0)) * sizeof(double);
     return p;
 }
-
-// whether a precision / shape order keeps the x-difference tile: FP64 linear
-__host__ __device__ inline bool uses_xdiff(int prec, int order) { return prec == 0 && order == 1; }
 
 // double <-> float on the bit patterns without branches: magnitudes below
 // 2^-100 (and zero) become a signed zero (an absolute error below 2^-100,
@@ -556,8 +626,6 @@ __device__ __forceinline__ double f64_of(float f) {
 __device__ __forceinline__ void red_f64(double* p, double v) {
     asm volatile("red.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v) : "memory");
 }
-__device__ __forceinline__ void jadd(double* p, double v) { red_f64(p, v); }
-__device__ __forceinline__ void jadd(double* p, dd v) { red_f64(p, dd_to_norm(v)); }
 __device__ __forceinline__ void jadd(double* p, float v) { red_f64(p, f64_of(v)); }
 
 // Where a tile's current goes: base points at component 0 of local node
@@ -600,53 +668,7 @@ __device__ __forceinline__ bool deposit(const SV& S, const JView& V,
         Dx12[l] = k12 * wx.DS[l];
         Dz12[l] = k12 * wz.DS[l];
     }
-    if constexpr (DIM == 3 && std::is_same<R, dd>::value) {
-        // float-float: one loop over the three currents (prefix axis a,
-        // transverse axes b < c), to keep the code small
-        R Ay[W], Dy12[W];
-#pragma unroll
-        for (int l = 0; l < W; ++l) {
-            Ay[l] = fma(half, wy.DS[l], wy.S0[l]);
-            Dy12[l] = k12 * wy.DS[l];
-        }
-        double* origin = V.base + (wz.base + lo) * sz + (wy.base + lo) * sy + (wx.base + lo);
-#pragma unroll 1
-        for (int a = 0; a < 3; ++a) {
-            const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
-            const int sa = pick3(a, 1, sy, sz), sb = pick3(b, 1, sy, sz), sc = pick3(c, 1, sy, sz);
-            const R cf = qw * pick3(a, jf[0], jf[1], jf[2]);
-            R Pf[W - 1], Ab[W], Ac[W], Db[W], Dc12[W];
-            R acc = A::c(0.0);
-#pragma unroll
-            for (int l = 0; l < W; ++l) {
-                if (l < W - 1) {
-                    acc = acc + pick3(a, wx.DS[l], wy.DS[l], wz.DS[l]);
-                    Pf[l] = cf * acc;
-                }
-                Ab[l] = b == 0 ? Ax[l] : Ay[l];
-                Db[l] = b == 0 ? wx.DS[l] : wy.DS[l];
-                Ac[l] = c == 1 ? Ay[l] : Az[l];
-                Dc12[l] = c == 1 ? Dy12[l] : Dz12[l];
-            }
-            double* Ja = origin + a * V.cs;
-#pragma unroll 1
-            for (int k = 0; k < W; ++k) {
-                R ack = Ac[0], dck = Dc12[0];
-#pragma unroll
-                for (int q = 1; q < W; ++q) {
-                    ack = k == q ? Ac[q] : ack;
-                    dck = k == q ? Dc12[q] : dck;
-                }
-#pragma unroll
-                for (int j = 0; j < W; ++j) {
-                    const R T = fma(Ab[j], ack, Db[j] * dck);
-                    double* row = Ja + k * sc + j * sb;
-#pragma unroll
-                    for (int l = 0; l < W - 1; ++l) jadd(row + l * sa, Pf[l] * T);
-                }
-            }
-        }
-    } else if constexpr (DIM == 3) {
+    if constexpr (DIM == 3) {
         R Ay[W];
 #pragma unroll
         for (int l = 0; l < W; ++l) Ay[l] = fma(half, wy.DS[l], wy.S0[l]);
@@ -743,22 +765,8 @@ __device__ __forceinline__ bool deposit(const SV& S, const JView& V,
 // the two nodes of the cell, DS = (-d, d) with d = f1 - f0, so the prefix sum
 // has one term and the transverse weight A_a A_b + DS_a DS_b / 12 is
 // A_a A_b +- d_a d_b / 12 (A = (1 - m, m), m = f0 + d/2).  Same weights as
-// deposit<R, DIM, 1, 2>, with fewer instructions.
-template <class R, int DIM, class SV>
-__device__ __forceinline__ void deposit_lin_incell_d(const SV& S, const JView& V,
-                                                     R qw, R vy, const R* jf, const Support<1, R>* n,
-                                                     const R* disp);
-
-template <class R, int DIM, class SV>
-__device__ __forceinline__ void deposit_lin_incell(const SV& S, const JView& V,
-                                                   R qw, R vy, const R* jf,
-                                                   const Support<1, R>* n, const Support<1, R>* m) {
-    const R disp[3] = {m[0].w[1] - n[0].w[1], m[1].w[1] - n[1].w[1], m[2].w[1] - n[2].w[1]};
-    deposit_lin_incell_d<R, DIM, SV>(S, V, qw, vy, jf, n, disp);
-}
-
-// the same deposit, given the in-cell displacement disp[a] = x^{n+1} - x^n
-// (cells) of each direction
+// deposit<R, DIM, 1, 2>, with fewer instructions, given the displacement
+// disp[a] = x^{n+1} - x^n (cells) of each direction.
 template <class R, int DIM, class SV>
 __device__ __forceinline__ void deposit_lin_incell_d(const SV& S, const JView& V,
                                                      R qw, R vy, const R* jf, const Support<1, R>* n,
@@ -773,29 +781,7 @@ __device__ __forceinline__ void deposit_lin_incell_d(const SV& S, const JView& V
     const R mx = fma(half, dx, n[0].w[1]), mz = fma(half, dz, n[2].w[1]);
     const R ax0 = one - mx, az0 = one - mz;
     const int bx = n[0].s + lo, bz = n[2].s + lo;
-    if constexpr (DIM == 3 && std::is_same<R, dd>::value) {
-        // float-float: one loop over the three currents (axis a, transverse b < c)
-        const R dy = disp[1];
-        const R my = fma(half, dy, n[1].w[1]);
-        const R ay0 = one - my;
-        const int by = n[1].s + lo;
-        double* origin = V.base + bz * sz + by * sy + bx;
-#pragma unroll 1
-        for (int a = 0; a < 3; ++a) {
-            const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
-            const int sb = pick3(b, 1, sy, sz), sc = pick3(c, 1, sy, sz);
-            const R db = b == 0 ? dx : dy, dc = c == 1 ? dy : dz;
-            const R mb = b == 0 ? mx : my, mc = c == 1 ? my : mz;
-            const R ab = b == 0 ? ax0 : ay0, ac = c == 1 ? ay0 : az0;
-            const R e = (db * dc) * k12;
-            const R pf = -((qw * pick3(a, jf[0], jf[1], jf[2])) * pick3(a, dx, dy, dz));
-            double* r = origin + a * V.cs;
-            jadd(r, pf * fma(ab, ac, e));
-            jadd(r + sb, pf * fma(mb, ac, -e));
-            jadd(r + sc, pf * fma(ab, mc, -e));
-            jadd(r + sb + sc, pf * fma(mb, mc, e));
-        }
-    } else if constexpr (DIM == 3) {
+    if constexpr (DIM == 3) {
         // value of node (b, c) of current a: pf_a (A_b A_c + s d_b d_c / 12),
         // s = +1 on the diagonal nodes, -1 off it, pf_a = -q w jf_a d_a; with
         // pe_a = pf_a d_b d_c / 12 = -q w jf_a (d_x d_y d_z / 12) and the node
@@ -860,6 +846,255 @@ __device__ __forceinline__ void deposit_lin_incell_d(const SV& S, const JView& V
     }
 }
 
+// ---- FP64: fixed-point Esirkepov deposit ----------------------------------
+// A contribution is amplitude x weight: the weight (the transverse factor, in
+// [0, 1]) is a Q62 number, the amplitude (prefactor, q w and the prefix sum of
+// DS along the current's direction, or v_y in 2D) an Amp; their product is
+// rounded once, to the double that goes to L2.  Against FP64 factors this takes
+// the deposit off the FP64 pipe (36 of about 165 FP64 instructions per particle
+// for linear shapes) and rounds each contribution once instead of four to six
+// times.
+//
+// T >= 0.  The contribution is rounded toward zero (at most 2^-52 of it, where
+// the FP64 factors took four to six roundings of 2^-53 each).
+__device__ __forceinline__ void emit(double* p, const Amp& a, q62 T) {
+    const u64 jm = mulhi(a.m, (u64)T);  // value jm 2^(e + 2)
+    if (jm != 0ull) red_f64(p, pack_double<false>(jm, a.es + (1087u << 20)));
+}
+// amplitudes whose contributions may leave the normal doubles: f, the product
+// of the FP64 factors, times the weight
+static __device__ __noinline__ void emit_any(double* p, double f, q62 T) {
+    red_f64(p, f * ((double)T * 2.168404344971009e-19));  // 2^-62
+}
+
+// node shapes of a move on a common window of W nodes: A = (S0 + S1) / 2,
+// D = S1 - S0
+template <int W>
+struct WindowQ {
+    int base;
+    q62 A[W], D[W];
+};
+template <int ORDER, int W>
+__device__ __forceinline__ bool make_window_q(const SupQ<ORDER>& a, const SupQ<ORDER>& b, WindowQ<W>& win) {
+    const int base = min(a.s, b.s);
+    const int oa = a.s - base, ob = b.s - base;
+    // unsigned: a cell index saturated by a move of 2^31 cells or more wraps the difference
+    if ((unsigned)oa > (unsigned)(W - ORDER - 1) || (unsigned)ob > (unsigned)(W - ORDER - 1)) return false;
+    win.base = base;
+#pragma unroll
+    for (int l = 0; l < W; ++l) {
+        q62 s0 = 0, s1 = 0;
+#pragma unroll
+        for (int k = 0; k <= ORDER; ++k) {
+            const q62 wa = ORDER == 1 && k == 0 ? kOneQ - a.w[ORDER] : a.w[k];
+            const q62 wb = ORDER == 1 && k == 0 ? kOneQ - b.w[ORDER] : b.w[k];
+            s0 = (l - oa == k) ? wa : s0;
+            s1 = (l - ob == k) ? wb : s1;
+        }
+        win.A[l] = (s0 + s1) >> 1;
+        win.D[l] = s1 - s0;
+    }
+    return true;
+}
+
+constexpr q62 kTwelfthQ = 384307168202282326ll;  // 2^62 / 12
+
+// Deposit on windows of W nodes per direction: for each current (a loop: one
+// copy of the code, whose size the instruction cache feels) the prefix sums of
+// D along its own direction times the transverse weight A_b A_c + D_b D_c / 12.
+// ANY: amplitudes of any size (emit_any).
+template <int DIM, int ORDER, int W, bool ANY>
+__device__ __forceinline__ bool deposit_q(int lo, const JView& V, const Amp* ja, const double* jf, double qw,
+                                          double vy, const SupQ<ORDER>* n, const SupQ<ORDER>* m) {
+    WindowQ<W> w0, w1, w2;
+    bool ok = make_window_q<ORDER, W>(n[0], m[0], w0) && make_window_q<ORDER, W>(n[2], m[2], w2);
+    if (DIM == 3) ok = ok && make_window_q<ORDER, W>(n[1], m[1], w1);
+    if (!ok) return false;
+    constexpr int UW = ANY ? 1 : W;                     // inner loops: unrolled, but for the rare case
+    constexpr int UK = ANY || ORDER > 1 ? 1 : W;        // outer transverse loop: rolled for long windows
+    double* origin = V.base + (w2.base + lo) * V.sz + (w0.base + lo);
+    if (DIM == 3) origin += (w1.base + lo) * V.sy;
+    const Amp q = amp_of(qw);
+    auto out = [&](double* p, const Amp& a, q62 T, double f) {
+        if constexpr (ANY) emit_any(p, f, T);
+        else emit(p, a, T);
+    };
+    if constexpr (DIM == 3) {
+#pragma unroll 1
+        for (int a = 0; a < 3; ++a) {
+            const int b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
+            const int sa = pick3(a, 1, V.sy, V.sz), sb = pick3(b, 1, V.sy, V.sz), sc = pick3(c, 1, V.sy, V.sz);
+            const Amp cw = amp_mul(pick3(a, ja[0], ja[1], ja[2]), q);
+            const double cf = ANY ? pick3(a, jf[0], jf[1], jf[2]) * qw : 0.0;
+            Amp pf[W - 1];
+            double nf[W - 1];
+            Limb Ab[W], Db[W], Ac[W], Dc[W];
+            q62 acc = 0;
+#pragma unroll
+            for (int l = 0; l < W; ++l) {
+                if (l < W - 1) {
+                    acc += pick3(a, w0.D[l], w1.D[l], w2.D[l]);
+                    pf[l] = amp_scale(cw, acc);
+                    nf[l] = ANY ? cf * ((double)acc * 2.168404344971009e-19) : 0.0;
+                }
+                Ab[l] = limb_of(b == 0 ? w0.A[l] : w1.A[l]);
+                Db[l] = limb_of(b == 0 ? w0.D[l] : w1.D[l]);
+                Ac[l] = limb_of(c == 1 ? w1.A[l] : w2.A[l]);
+                Dc[l] = limb_of(mulq(limb_of(c == 1 ? w1.D[l] : w2.D[l]), limb_of(kTwelfthQ)));
+            }
+            double* Ja = origin + a * V.cs;
+#pragma unroll UK
+            for (int k = 0; k < W; ++k) {
+                Limb ak = Ac[0], dk = Dc[0];
+#pragma unroll
+                for (int i = 1; i < W; ++i) {
+                    ak = k == i ? Ac[i] : ak;
+                    dk = k == i ? Dc[i] : dk;
+                }
+                double* plane = Ja + k * sc;
+#pragma unroll UW
+                for (int j = 0; j < W; ++j) {
+                    AccQ s;
+                    s.mac(Ab[j], ak);
+                    s.mac(Db[j], dk);
+                    const q62 T = max(s.get(), 0ll);
+                    double* row = plane + j * sb;
+#pragma unroll UW
+                    for (int l = 0; l < W - 1; ++l) out(row + l * sa, pf[l], T, nf[l]);
+                }
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (int a = 0; a < 2; ++a) {  // Jx, then Jz: the transverse weight is A
+            const int sa = a == 0 ? 1 : V.sz, sb = a == 0 ? V.sz : 1;
+            const Amp cw = amp_mul(a == 0 ? ja[0] : ja[2], q);
+            const double cf = ANY ? (a == 0 ? jf[0] : jf[2]) * qw : 0.0;
+            double* Ja = origin + (a == 0 ? 0 : 2 * V.cs);
+            q62 acc = 0;
+#pragma unroll UW
+            for (int l = 0; l < W - 1; ++l) {
+                acc += a == 0 ? w0.D[l] : w2.D[l];
+                const Amp pf = amp_scale(cw, acc);
+                const double nf = ANY ? cf * ((double)acc * 2.168404344971009e-19) : 0.0;
+#pragma unroll UW
+                for (int j = 0; j < W; ++j) out(Ja + j * sb + l * sa, pf, a == 0 ? w2.A[j] : w0.A[j], nf);
+            }
+        }
+        // out-of-plane Jy = q w vy / (dx dz) (Ax Az + Dx Dz / 12)
+        const Amp cv = amp_mul(amp_mul(ja[1], q), amp_of(vy));
+        const double nfy = ANY ? jf[1] * qw * vy : 0.0;
+        double* Jy = origin + V.cs;
+#pragma unroll UW
+        for (int k = 0; k < W; ++k) {
+            const Limb ak = limb_of(w2.A[k]), dk = limb_of(mulq(limb_of(w2.D[k]), limb_of(kTwelfthQ)));
+#pragma unroll UW
+            for (int i = 0; i < W; ++i) {
+                AccQ s;
+                s.mac(limb_of(w0.A[i]), ak);
+                s.mac(limb_of(w0.D[i]), dk);
+                out(Jy + k * V.sz + i, cv, max(s.get(), 0ll), nfy);
+            }
+        }
+    }
+    return true;
+}
+
+// whether every amplitude of a particle stays inside the normal doubles (a zero
+// q w or v_y deposits nothing, and is)
+template <int DIM>
+__device__ __forceinline__ bool amps_safe(const ExpRange& r, double qw, double vy) {
+    const int eq = exp_field(qw);
+    bool ok = in_range(r, eq);
+    if (DIM == 2) {
+        const int ev = exp_field(vy);
+        ok = ok && (vy == 0.0 || (ev > 0 && ev < 0x7FF && in_range(r, eq + ev - 1023)));
+    }
+    return ok || qw == 0.0;
+}
+
+// Linear shapes, particle keeping its cell: the window is the two nodes of the
+// cell, D = (-d, d), one prefix sum, and with the mid-path offsets m and
+// P = m_b m_c + d_b d_c / 12 the four weights are P, m_b - P, m_c - P and
+// 1 - m_b - m_c + P.  cw: prefactor x q w per current (2D: x v_y for y).  P
+// comes out up to 5 units of 2^-62 low: it is raised by 6 and m_b, m_c (by a
+// half low themselves) by 8, so that no weight is negative.
+template <int DIM>
+__device__ __forceinline__ void deposit_lin_q(int lo, const JView& V, const Amp* cw, const SupQ<1>* n,
+                                              const SupQ<1>* mv) {
+    q62 d[3], m[3];
+    Limb lm[3], l12[3], ld[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (DIM == 2 && a == 1) continue;
+        d[a] = mv[a].w[1] - n[a].w[1];
+        const q62 h = (n[a].w[1] + mv[a].w[1]) >> 1;
+        m[a] = h + 8;
+        lm[a] = limb_of(h);
+        ld[a] = limb_of(d[a]);
+        if (a > 0) l12[a] = limb_of(mulq(ld[a], limb_of(kTwelfthQ)));
+    }
+    double* origin = V.base + (n[2].s + lo) * V.sz + (n[0].s + lo);
+    if (DIM == 3) origin += (n[1].s + lo) * V.sy;
+    auto four = [&](double* r, const Amp& pf, q62 mb, q62 mc, const Limb& lb, const Limb& lc, const Limb& db,
+                    const Limb& dc12, int sb, int sc) {
+        AccQ s;
+        s.mac(lb, lc);
+        s.mac(db, dc12);
+        const q62 P = s.get() + 6;
+        emit(r, pf, kOneQ + 16 - mb - mc + P);
+        emit(r + sb, pf, mb - P);
+        emit(r + sc, pf, mc - P);
+        emit(r + sb + sc, pf, P);
+    };
+    if constexpr (DIM == 3) {
+        // a loop: the instruction cache feels three copies (128^3 foil 1567 -> 1524 us)
+#pragma unroll 1
+        for (int a = 0; a < 3; ++a) {
+            const Amp pf = amp_scale(pick3(a, cw[0], cw[1], cw[2]), -pick3(a, d[0], d[1], d[2]));
+            four(origin + a * V.cs, pf, a == 0 ? m[1] : m[0], a == 2 ? m[1] : m[2], a == 0 ? lm[1] : lm[0],
+                 a == 2 ? lm[1] : lm[2], a == 0 ? ld[1] : ld[0], a == 2 ? l12[1] : l12[2], a == 0 ? V.sy : 1,
+                 a == 2 ? V.sy : V.sz);
+        }
+    } else {
+        const Amp px = amp_scale(cw[0], -d[0]), pz = amp_scale(cw[2], -d[2]);
+        emit(origin, px, kOneQ + 8 - m[2]);
+        emit(origin + V.sz, px, m[2]);
+        emit(origin + 2 * V.cs, pz, kOneQ + 8 - m[0]);
+        emit(origin + 2 * V.cs + 1, pz, m[0]);
+        four(origin + V.cs, cw[1], m[0], m[2], lm[0], lm[2], ld[0], l12[2], 1, V.sz);
+    }
+}
+
+// node supports of a move, from the positions
+template <int DIM, int ORDER>
+__device__ __forceinline__ void node_supports_q(const double* x, const int* o, SupQ<ORDER>* n, bool& nan) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (DIM == 2 && a == 1) continue;
+        const CellQ c = cell_q(x[a]);
+        nan = nan || c.nan;
+        n[a] = node_support<ORDER>(c, o[a]);
+    }
+}
+
+// any particle's deposit on the ORDER + 2 window with amplitudes of any size
+// (weights or prefactors near the ends of the double range, Inf, NaN)
+template <int DIM, int ORDER>
+static __device__ __noinline__ bool deposit_any(const SimDev& S, JView V, int ox, int oy, int oz, double X, double Y,
+                                                double Z, double X1, double Y1, double Z1, double qw, double vy) {
+    const int o[3] = {ox, oy, oz};
+    const double x0[3] = {X, Y, Z}, x1[3] = {X1, Y1, Z1};
+    const double jf[3] = {S.jfac[0], DIM == 3 ? S.jfac[1] : S.jyfac2d, S.jfac[2]};
+    const Amp ja[3] = {amp_of(jf[0]), amp_of(jf[1]), amp_of(jf[2])};
+    SupQ<ORDER> n[3], m[3];
+    bool nan = false;
+    node_supports_q<DIM, ORDER>(x0, o, n, nan);
+    node_supports_q<DIM, ORDER>(x1, o, m, nan);
+    return deposit_q<DIM, ORDER, ORDER + 2, true>(S.jlo, V, ja, jf, nan ? qw * __longlong_as_double(0x7FF8000000000000ll) : qw,
+                                                  vy, n, m);
+}
+
 // One particle's stored state as read from HBM (positions in global cell
 // units, momenta and weight as stored); loaded ahead of its push so that the
 // loads of several particles per thread can be in flight together.
@@ -901,13 +1136,153 @@ __device__ __forceinline__ PIn read_staged(const double* slot) {
     return in;
 }
 
-// Gather, Boris push, and deposit of one particle.  Particles that keep their
+// Gather, Boris push, and deposit of one particle, FP64.  The gather and the
+// deposit are fixed-point; fx: the staged tile is in fixed point (emax: biased
+// exponents per component), otherwise it holds the doubles as loaded.
+template <class R, int DIM, int ORDER, class SV, class SPV>
+__device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const SimDev& SG, const Tile& tl,
+                                           const double* __restrict__ sEB, bool fx, const int* __restrict__ emax,
+                                           const JView& V, double* __restrict__ sQw, unsigned* s_tail,
+                                           const SmemPlan& P, const R* dtd, R kq, double qs, int64_t p, const PIn& in,
+                                           int32_t* err) {
+    using A = Arith<R>;
+    const double x0[3] = {in.X, DIM == 3 ? in.Y : 0.0, in.Z};
+    double qw = qs * in.w;
+
+    // ---- gather at x^n: node and half-node supports per direction (tile-local nodes)
+    SupQ<ORDER> nd[3];
+    Six f;
+    {
+        AxisQ<ORDER> na[3], ha[3];
+        bool inside = true, nan = false;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (DIM == 2 && a == 1) continue;
+            const CellQ c = cell_q(x0[a]);
+            nan = nan || c.nan;
+            inside = inside && (unsigned)(c.i - tl.o[a]) < (unsigned)S.T[a];
+            nd[a] = node_support<ORDER>(c, tl.o[a]);
+            na[a] = axis_of<ORDER>(nd[a]);
+            ha[a] = axis_of<ORDER>(half_support<ORDER>(c, tl.o[a], S.ec != 0));
+        }
+        if (!inside) {
+            // the particle must sit in its tile; the E/B halo then covers every support above
+            atomicOr(err, PIC_DERR_BOUNDS);
+            sp.key[p] = S.ntiles;
+            warp_hist_add(sp.count, S.ntiles);
+            return;
+        }
+        if (fx)
+            f = gather6_q<ORDER, DIM>(reinterpret_cast<const long long*>(sEB), P.eb_stride, S.ebs[0], S.ebs[1], emax,
+                                      na, ha);
+        else
+            f = gather6_fp64<ORDER, DIM>(sEB, P.eb_stride, S.ebs[0], S.ebs[1], x0[0], x0[1], x0[2], tl.o[0], tl.o[1],
+                                         tl.o[2], S.ec != 0);
+        if (nan) f.v[0] = f.v[1] = f.v[2] = __longlong_as_double(0x7FF8000000000000ll);
+    }
+    const R u0 = A::from(in.u0), u1 = A::from(in.u1), u2 = A::from(in.u2);
+    const R e0 = A::from(f.v[0]), e1 = A::from(f.v[1]), e2 = A::from(f.v[2]);
+    const R b0 = A::from(f.v[3]), b1 = A::from(f.v[4]), b2 = A::from(f.v[5]);
+
+    // ---- relativistic Boris push
+    const R one = A::c(1.0);
+    const R m0 = fma(kq, e0, u0), m1 = fma(kq, e1, u1), m2 = fma(kq, e2, u2);
+    const R ig = A::rsqrt(fma(m2, m2, fma(m1, m1, fma(m0, m0, one))));
+    const R kg = kq * ig;
+    const R t0 = kg * b0, t1 = kg * b1, t2 = kg * b2;
+    const R sf = A::two_over(fma(t2, t2, fma(t1, t1, fma(t0, t0, one))));
+    const R s0 = sf * t0, s1 = sf * t1, s2 = sf * t2;
+    // u' = u- + u- x t, u+ = u- + u' x s, each component as two FMAs
+    const R d0 = fma(m1, t2, fma(-m2, t1, m0));
+    const R d1 = fma(m2, t0, fma(-m0, t2, m1));
+    const R d2 = fma(m0, t1, fma(-m1, t0, m2));
+    const R p0 = fma(d1, s2, fma(-d2, s1, m0));
+    const R p1 = fma(d2, s0, fma(-d0, s2, m1));
+    const R p2 = fma(d0, s1, fma(-d1, s0, m2));
+    const R n0 = fma(kq, e0, p0), n1 = fma(kq, e1, p1), n2 = fma(kq, e2, p2);
+    const R ign = A::rsqrt(fma(n2, n2, fma(n1, n1, fma(n0, n0, one))));
+    const R v1 = n1 * ign;
+    double x1[3];
+    x1[0] = A::move(n0 * ign, dtd[0], x0[0]);
+    x1[1] = DIM == 3 ? A::move(v1, dtd[1], x0[1]) : 0.0;
+    x1[2] = A::move(n2 * ign, dtd[2], x0[2]);
+    const double vy = DIM == 3 ? 0.0 : A::to(v1);
+
+    // ---- Esirkepov deposit of J^{n+1/2} from x^n to x^{n+1}
+    SupQ<ORDER> mv[3];
+    int g[3] = {0, 0, 0};
+    bool same = true, nan = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (DIM == 2 && a == 1) continue;
+        const CellQ c = cell_q(x1[a]);
+        nan = nan || c.nan;
+        g[a] = c.i;
+        mv[a] = node_support<ORDER>(c, tl.o[a]);
+        same = same && mv[a].s == nd[a].s;
+    }
+    if (nan) qw = __longlong_as_double(0x7FF8000000000000ll);
+    if (same) {
+        const bool ok = amps_safe<DIM>(S.je, qw, vy);
+        if constexpr (ORDER == 1) {
+            if (ok) {
+                const Amp q = amp_of(qw);
+                Amp cw[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) cw[a] = amp_mul(S.ja[a], q);
+                if (DIM == 2) cw[1] = amp_mul(cw[1], amp_of(vy));
+                deposit_lin_q<DIM>(S.jlo, V, cw, nd, mv);
+            }
+        } else {
+            if (ok) deposit_q<DIM, ORDER, ORDER + 1, false>(S.jlo, V, S.ja, nullptr, qw, vy, nd, mv);
+        }
+        if (!ok)
+            deposit_any<DIM, ORDER>(SG, V, tl.o[0], tl.o[1], tl.o[2], x0[0], x0[1], x0[2], x1[0], x1[1], x1[2], qw, vy);
+    } else {
+        // the ring never holds more than 31 + 32 entries: the warp drains 32
+        // whenever 32 are waiting
+        const unsigned slot = atomicAdd(s_tail, 1u) & (WQ - 1);
+        sQw[0 * WQ + slot] = x0[0];
+        sQw[1 * WQ + slot] = x0[2];
+        sQw[2 * WQ + slot] = x1[0];
+        sQw[3 * WQ + slot] = x1[2];
+        sQw[4 * WQ + slot] = qw;
+        sQw[5 * WQ + slot] = DIM == 3 ? x0[1] : vy;
+        if (DIM == 3) sQw[6 * WQ + slot] = x1[1];
+    }
+
+    // ---- new position, boundary, re-sort key
+    auto wrap = [&](int a) {
+        if (is_neg(x1[a]) || ge_pos(x1[a], S.nd[a])) x1[a] = wrap_periodic(x1[a], S.nd[a]);
+    };
+    const int r[3] = {g[0] - tl.o[0], g[1] - tl.o[1], g[2] - tl.o[2]};
+    int key = near_key<DIM>(S, S.nk, r);
+    // z < A or z >= n - A for integer bounds: compare floor(z)
+    if (S.absorb > 0 && (g[2] < S.absorb || g[2] >= S.n[2] - S.absorb)) key = S.ntiles;
+    wrap(0);
+    if (DIM == 3) wrap(1);
+    if (S.absorb <= 0) wrap(2);
+    if (key < 0) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) g[a] = DIM == 3 || a != 1 ? min(max(ifloor(x1[a]), 0), S.n[a] - 1) : 0;
+        key = tile_key(S, g[0], g[1], g[2]);
+    }
+    sp.cur[0][p] = x1[0];
+    if (DIM == 3) sp.cur[1][p] = x1[1];
+    sp.cur[2][p] = x1[2];
+    sp.cur[3][p] = A::to(n0);
+    sp.cur[4][p] = A::to(n1);
+    sp.cur[5][p] = A::to(n2);
+    sp.key[p] = key;
+    warp_hist_add(sp.count, key);
+}
+
+// The same in FP32 (R = float), quadratic and cubic shapes.  Particles that keep their
 // support in every direction deposit at once on the small window; the others
 // go to the warp's ring buffer, drained 32 at a time by drain_warp.
 template <class R, int DIM, int ORDER, class SV, class SPV>
 __device__ __forceinline__ void push_one(const SV& S, const SPV& sp, const Tile& tl,
-                                         const R* __restrict__ sEB, const R* __restrict__ sD,
-                                         const JView& V,
+                                         const R* __restrict__ sEB, const JView& V,
                                          double* __restrict__ sQw, unsigned* s_tail, const SmemPlan& P,
                                          const R* jf, const R* dtd, R kq, R qs, int64_t p, const PIn& in,
                                          int32_t* err) {
@@ -944,7 +1319,7 @@ __device__ __forceinline__ void push_one(const SV& S, const SPV& sp, const Tile&
     }
     const int SX = S.ebs[0], SY = S.ebs[1];
     R ev[3], bv[3];
-    gather6<R, ORDER, DIM>(sEB, P.eb_stride, SX, SY, nd, hf, ev, bv, sD, P.d_stride);
+    gather6<R, ORDER, DIM>(sEB, P.eb_stride, SX, SY, nd, hf, ev, bv);
     const R e0 = ev[0], e1 = ev[1], e2 = ev[2], b0 = bv[0], b1 = bv[1], b2 = bv[2];
 
     // ---- relativistic Boris push
@@ -979,10 +1354,7 @@ __device__ __forceinline__ void push_one(const SV& S, const SPV& sp, const Tile&
     else mv[1] = nd[1];
     bool same = mv[0].s == nd[0].s && mv[2].s == nd[2].s && (DIM == 2 || mv[1].s == nd[1].s);
     if (same) {
-        if constexpr (ORDER == 1)
-            deposit_lin_incell<R, DIM, SV>(S, V, qw, v1, jf, nd, mv);
-        else
-            deposit<R, DIM, ORDER, ORDER + 1>(S, V, qw, v1, jf, nd[0], nd[1], nd[2], mv[0], mv[1], mv[2]);
+        deposit<R, DIM, ORDER, ORDER + 1>(S, V, qw, v1, jf, nd[0], nd[1], nd[2], mv[0], mv[1], mv[2]);
     } else {
         // the ring never holds more than 31 + 32 entries: the warp drains 32
         // whenever 32 are waiting
@@ -1193,6 +1565,7 @@ __device__ __forceinline__ void push_one_f32lin(const SV& S, const SPV& sp, cons
     // new position, boundary, re-sort key
     double X = unfix24(b1[0]), Y = DIM == 3 ? unfix24(b1[1]) : 0.0, Z = unfix24(b1[2]);
     int g[3] = {(int)(b1[0] >> 24), DIM == 3 ? (int)(b1[1] >> 24) : 0, (int)(b1[2] >> 24)};
+    const int rel[3] = {g[0] - tl.o[0], g[1] - tl.o[1], g[2] - tl.o[2]};
     if (g[0] < 0 || g[0] >= S.n[0]) {
         X = wrap_periodic(X, S.nd[0]);
         g[0] += g[0] < 0 ? S.n[0] : -S.n[0];
@@ -1209,11 +1582,10 @@ __device__ __forceinline__ void push_one_f32lin(const SV& S, const SPV& sp, cons
         g[2] += g[2] < 0 ? S.n[2] : -S.n[2];
     }
     if (key < 0) {
-        bool own = (unsigned)(g[0] - tl.o[0]) < (unsigned)S.T[0] && (unsigned)(g[2] - tl.o[2]) < (unsigned)S.T[2];
-        if (DIM == 3) own = own && (unsigned)(g[1] - tl.o[1]) < (unsigned)S.T[1];
-        key = own ? tl.t
-                  : tile_key(S, min(max(g[0], 0), S.n[0] - 1), DIM == 3 ? min(max(g[1], 0), S.n[1] - 1) : 0,
-                             min(max(g[2], 0), S.n[2] - 1));
+        key = near_key<DIM>(S, S.nk, rel);
+        if (key < 0)
+            key = tile_key(S, min(max(g[0], 0), S.n[0] - 1), DIM == 3 ? min(max(g[1], 0), S.n[1] - 1) : 0,
+                           min(max(g[2], 0), S.n[2] - 1));
     }
     sp.cur[0][p] = X;
     if (DIM == 3) sp.cur[1][p] = Y;
@@ -1261,25 +1633,39 @@ __device__ __forceinline__ void drain_warp(const SimDev& S, const Tile& tl,
         atomicOr(err, PIC_DERR_BOUNDS);
 }
 
-// float-float keeps the drain out of line: the cell-crossing deposit is long
-// and rare, and inlined into the particle loop it crowds the instruction cache
-// (about 5 % of the kernel); FP64 is indifferent and inlines it, as does FP32
-template <class R, int DIM, int ORDER>
-__device__ __noinline__ void drain_warp_outlined(const SimDev& S, const Tile& tl,
-                                                 const JView& V,
-                                                 const double* __restrict__ sQw, unsigned head, unsigned n,
-                                                 const R* jf, int32_t* err) {
-    drain_warp<R, DIM, ORDER>(S, tl, V, sQw, head, n, jf, err);
+// the same in FP64: fixed-point deposit
+template <int DIM, int ORDER>
+__device__ __noinline__ void drain_warp_q(const SimDev& S, const Tile& tl, const JView& V,
+                                             const double* __restrict__ sQw, unsigned head, unsigned n,
+                                             int32_t* err) {
+    const unsigned lane = threadIdx.x & 31u;
+    if (lane >= n) return;
+    const unsigned i = (head + lane) & (WQ - 1);
+    const double x0[3] = {sQw[0 * WQ + i], DIM == 3 ? sQw[5 * WQ + i] : 0.0, sQw[1 * WQ + i]};
+    const double x1[3] = {sQw[2 * WQ + i], DIM == 3 ? sQw[6 * WQ + i] : 0.0, sQw[3 * WQ + i]};
+    const double qw = sQw[4 * WQ + i], vy = DIM == 3 ? 0.0 : sQw[5 * WQ + i];
+    const Amp ja[3] = {amp_of(S.jfac[0]), amp_of(DIM == 3 ? S.jfac[1] : S.jyfac2d), amp_of(S.jfac[2])};
+    bool ok;
+    if (amps_safe<DIM>(exp_range(S.jfac[0], DIM == 3 ? S.jfac[1] : S.jyfac2d, S.jfac[2]), qw, vy)) {
+        SupQ<ORDER> nd[3], mv[3];
+        bool nan = false;  // a NaN position comes with a NaN qw, which is not safe
+        node_supports_q<DIM, ORDER>(x0, tl.o, nd, nan);
+        node_supports_q<DIM, ORDER>(x1, tl.o, mv, nan);
+        ok = deposit_q<DIM, ORDER, ORDER + 2, false>(S.jlo, V, ja, nullptr, qw, vy, nd, mv);
+    } else {
+        ok = deposit_any<DIM, ORDER>(S, V, tl.o[0], tl.o[1], tl.o[2], x0[0], x0[1], x0[2], x1[0], x1[1], x1[2], qw, vy);
+    }
+    if (!ok) atomicOr(err, PIC_DERR_BOUNDS);
 }
 
 template <class R, int DIM, int ORDER>
 __device__ __forceinline__ void drain(const SimDev& S, const Tile& tl, const JView& V,
                                       const double* __restrict__ sQw, unsigned head, unsigned n,
                                       const R* jf, int32_t* err) {
-    if constexpr (!std::is_same<R, dd>::value)
+    if constexpr (std::is_same<R, float>::value)
         drain_warp<R, DIM, ORDER>(S, tl, V, sQw, head, n, jf, err);
     else
-        drain_warp_outlined<R, DIM, ORDER>(S, tl, V, sQw, head, n, jf, err);
+        drain_warp_q<DIM, ORDER>(S, tl, V, sQw, head, n, err);
 }
 
 // the J view of tile tl: the global padded arrays
@@ -1316,8 +1702,8 @@ struct SimConsts {
 
 // MINB = resident CTAs per SM the register allocation is sized for (1: up to
 // 255 registers, 8 warps per SM; 2: at most 128 registers, 16 warps per SM).
-// PREC = arithmetic of the particle push: 0 FP64, 1 float-float, 2 FP32 (storage,
-// positions and index math stay FP64 in all three, and the current goes to the
+// PREC = arithmetic of the particle push: 0 FP64, 2 FP32 (storage,
+// positions and index math stay FP64 in both, and the current goes to the
 // global FP64 J by L2 reductions).
 // PPT = particles per thread per loop iteration: their HBM loads are issued
 // together before the first of them is pushed (FP32 with PPT 1 stages each
@@ -1325,19 +1711,17 @@ struct SimConsts {
 template <int DIM, int ORDER, int MINB, int PREC, int PPT>
 __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev* __restrict__ sd,
                                                               SimDev* __restrict__ sims) {
-    using R = typename std::conditional<PREC == 1, dd, typename std::conditional<PREC == 2, float, double>::type>::type;
+    using R = typename std::conditional<PREC == 2, float, double>::type;
     using A = Arith<R>;
-    constexpr bool XD = PREC == 0 && ORDER == 1;  // x-difference tile beside the E/B tile
-    constexpr bool FC = PREC == 2;                // E/B tile converted to floats in place; particle staging
     extern __shared__ __align__(128) double smem_raw[];
     __shared__ __align__(8) uint64_t bar;
     // TMA destinations must be 128-byte aligned: round the dynamic base up
-    double* smem = reinterpret_cast<double*>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
-    __shared__ int s_unit, s_list, s_abort;
+    double* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 127u) / sizeof(double);
+    __shared__ int s_unit, s_list, s_abort, s_tile0, s_tile1;
     __shared__ HotSim s_hot;
     __shared__ unsigned s_qhead[QMAXWARPS], s_qtail[QMAXWARPS];
-    __shared__ unsigned long long s_cost;
+    __shared__ unsigned long long s_cost, s_time;
+    __shared__ int s_emax[6];  // fixed-point tile: biased exponent of each component's largest magnitude
 
     const int nlists = sd->meta[0];
     const int steal = sd->meta[1];
@@ -1347,14 +1731,15 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
         s_list = my_list;
         s_abort = 0;
         for (int w = 0; w < QMAXWARPS; ++w) s_qhead[w] = s_qtail[w] = 0u;
-        s_cost = 0ull;
+        s_cost = s_time = 0ull;
     }
     __syncthreads();
     uint32_t phase = 0;
     Tile cur;
     cur.sim = -1;
     cur.t = -1;
-    int visited = 0;
+    int visited = 0, hot = -1;
+    bool fx = false;  // the staged tile is in fixed point
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // ring of cell-crossing particles, in global scratch (L1/L2 resident; a
     // drain runs once per 32 crossings)
@@ -1388,8 +1773,8 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                 ++visited;
             }
             s_unit = u;
-            // every warp has left the previous unit (its closing barrier): restage
-            if (u >= 0) stage_hot(s_hot, sims[sd->units[u].sim]);
+            s_tile0 = 0x7FFFFFFF;
+            s_tile1 = -1;
         }
         __syncthreads();
         const int u = s_unit;
@@ -1397,27 +1782,50 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
         const UnitDev unit = sd->units[u];
         const SimDev& S = sims[unit.sim];
         const bool cap_clk = (S.capture & 1) != 0, cap_time = (S.capture & 2) != 0;
-        const uint64_t t_unit0 = (threadIdx.x == 0 && cap_time) ? globaltimer() : 0ull;
-        const SmemPlan P = smem_plan(S.ebs, XD, FC);
+        const SmemPlan P = smem_plan(S.ebs);
         double* sEBd = smem;
-        double* sDd = smem + 6 * P.eb_stride;   // x differences (linear FP64)
         const R* sEB = reinterpret_cast<const R*>(smem);
         unsigned long long my_clk = 0ull;
         const SimConsts<R, DIM> K(S);
+        const int t_first = unit.box * S.tiles_per_box;
+        const int t_end = t_first + S.tiles_per_box;
 
-        for (int spi = 0; spi < S.nsp; ++spi) {
-            const SpeciesDev& sp = S.sp[spi];
-            const R kq = A::from(sp.kq);
-            const R qs = A::from(sp.q);
-            const int t_first = unit.box * S.tiles_per_box;
-            const int t_end = t_first + S.tiles_per_box;
-            const int64_t b0 = sp.off[t_first], nbp = sp.off[t_end] - b0;
-            const int64_t r0 = b0 + (nbp * unit.chunk) / unit.nchunks;
-            const int64_t r1 = b0 + (nbp * (unit.chunk + 1)) / unit.nchunks;
-            if (r0 >= r1) continue;
-            for (int t = t_first; t < t_end; ++t) {
-                const int64_t s0 = max(sp.off[t], r0), s1 = min(sp.off[t + 1], r1);
-                if (s0 >= s1) continue;
+        // the unit's particle range of each species, and the tiles it touches
+        if (unit.sim != hot) {
+            stage_hot(s_hot, S);
+            hot = unit.sim;
+        }
+        {
+            const int i = (int)threadIdx.x - 4;
+            if (i >= 0 && i < S.nsp) {
+                const SpeciesDev& sp = S.sp[i];
+                const int64_t b0 = sp.off[t_first], nbp = sp.off[t_end] - b0;
+                s_hot.sp[i].r0 = b0 + (nbp * unit.chunk) / unit.nchunks;
+                s_hot.sp[i].r1 = b0 + (nbp * (unit.chunk + 1)) / unit.nchunks;
+            }
+        }
+        __syncthreads();
+        const int nsp = s_hot.nsp;
+        for (int i = threadIdx.x; i < nsp * S.tiles_per_box; i += blockDim.x) {
+            const int spi = i / S.tiles_per_box, t = t_first + i - spi * S.tiles_per_box;
+            const HotSp& sp = s_hot.sp[spi];
+            if (max(sp.off[t], sp.r0) < min(sp.off[t + 1], sp.r1)) {
+                atomicMin(&s_tile0, t);
+                atomicMax(&s_tile1, t);
+            }
+        }
+        __syncthreads();
+        uint64_t my_ns = 0ull;  // lane 0: ns of this warp's particle loops
+        // tile by tile, the species inside: a tile is staged once for all of them
+        {
+            const int t1 = s_tile1;
+            for (int t = s_tile0; t <= t1; ++t) {
+                bool any = false;
+                for (int spi = 0; spi < nsp; ++spi) {
+                    const HotSp& sp = s_hot.sp[spi];
+                    any = any || max(sp.off[t], sp.r0) < min(sp.off[t + 1], sp.r1);
+                }
+                if (!any) continue;
                 if (t != cur.t || unit.sim != cur.sim) {
                     if (cur.t >= 0 && unit.sim != cur.sim) drain_ring(sims[cur.sim]);
                     __syncthreads();
@@ -1425,6 +1833,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     cur.t = t;
                     tile_origin(S, t, cur.o);
                     if (threadIdx.x == 0) {
+                        for (int c = 0; c < 6; ++c) s_emax[c] = 0;
                         fence_proxy_async();
                         mbar_expect_tx(&bar, (uint32_t)(6 * P.eb_vol * sizeof(double)));
                         constexpr int H = EBHalo<ORDER>::lo;
@@ -1434,6 +1843,11 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
 #pragma unroll
                         for (int c = 0; c < 6; ++c)
                             tma_load_3d(sEBd + c * P.eb_stride, &S.tmap[c], x0, y0, z0, &bar);
+                    }
+                    for (int i = threadIdx.x; i < 9; i += blockDim.x) {
+                        const int a = i / 3, side = i - 3 * a;
+                        const int c = a == 0 ? cur.o[0] : (a == 1 ? cur.o[1] : cur.o[2]);
+                        s_hot.nk[a][side] = DIM == 2 && a == 1 ? 0 : key_part(s_hot, a, side == 0 ? c - 1 : (side == 1 ? c : c + s_hot.T[a]));
                     }
                     bool ok = mbar_wait_bounded(&bar, phase);
                     phase ^= 1u;
@@ -1448,28 +1862,29 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         __syncthreads();
                         return;
                     }
-                    if constexpr (XD) {
-                        // x differences of every staged row (each x lerp of the gather
-                        // becomes one FMA): one thread per row, walking along x
-                        const int SX = S.ebs[0], rows = S.ebs[1] * S.ebs[2];
-                        for (int i = threadIdx.x; i < 6 * rows; i += blockDim.x) {
-                            const int c = i / rows, row = i - c * rows;
-                            const double* f = sEBd + c * P.eb_stride + row * SX;
-                            double* dst = sDd + c * P.d_stride + row * (SX - 1);
-                            double prev = f[0];
-                            for (int x = 1; x < SX; ++x) {
-                                const double v = f[x];
-                                dst[x - 1] = v - prev;
-                                prev = v;
-                            }
+                    if constexpr (PREC != 2) {
+                        // E/B tile to fixed point in place: the exponent of each
+                        // component's largest magnitude, then the values in its units
+                        for (int c = 0; c < 6; ++c) {
+                            unsigned mx = 0u;
+#pragma unroll 4
+                            for (int i = threadIdx.x; i < P.eb_vol; i += blockDim.x)
+                                mx = max(mx, (unsigned)__double2hiint(sEBd[c * P.eb_stride + i]) & 0x7FFFFFFFu);
+                            mx = __reduce_max_sync(0xffffffffu, mx);
+                            if (lane == 0) atomicMax(&s_emax[c], (int)(mx >> 20));
                         }
                         __syncthreads();
-                    }
-                    if constexpr (PREC == 1) {
-                        // E/B tile to float pairs, in place (8 bytes either way)
-                        for (int i = threadIdx.x; i < 6 * P.eb_stride; i += blockDim.x) {
-                            const dd v = dd_from(sEBd[i]);
-                            reinterpret_cast<dd*>(sEBd)[i] = v;
+                        fx = true;
+                        for (int c = 0; c < 6; ++c) fx = fx && tile_exp_ok(s_emax[c]);
+                        if (fx) {
+                            for (int c = 0; c < 6; ++c) {
+                                const int em = s_emax[c];
+#pragma unroll 4
+                                for (int i = threadIdx.x; i < P.eb_vol; i += blockDim.x) {
+                                    double* v = sEBd + c * P.eb_stride + i;
+                                    *v = __longlong_as_double(tile_fix<TileBits<ORDER>::FB>(*v, em));
+                                }
+                            }
                         }
                         __syncthreads();
                     }
@@ -1507,19 +1922,38 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         __syncthreads();
                     }
                 }
+                const uint64_t t0 = lane == 0 && cap_time ? globaltimer() : 0ull;
                 const unsigned long long c0 = cap_clk ? clock64() : 0ull;
-                {
+                // groups of particles go round the warps, on across the species
+                const int nw = blockDim.x >> 5;
+                int turn = warp;
+                for (int spi = 0; spi < nsp; ++spi) {
                     // per-warp loop: no CTA barrier until the tile changes
+                    const HotSp& hs = s_hot.sp[spi];
+                    const int64_t s0 = max(hs.off[t], hs.r0), s1 = min(hs.off[t + 1], hs.r1);
+                    if (s0 >= s1) continue;
+                    const R kq = A::from(hs.kq);
+                    const R qs = A::from(hs.q);
+                    const double qsd = hs.q;
+                    const int64_t first = s0 + turn * (32 * PPT);
+                    {
+                        // this warp's place in the round after the species' last group
+                        const int ng = (int)((s1 - s0 + 32 * PPT - 1) / (32 * PPT));
+                        turn = (turn - ng) % nw;
+                        if (turn < 0) turn += nw;
+                    }
                     const JView V = j_view(S, cur);
                     double* sQw = gring;
-                    const R* sD = XD ? reinterpret_cast<const R*>(sDd) : nullptr;
                     volatile unsigned* vtail = s_qtail + warp;
                     auto push = [&](int64_t p, const PIn& in) {
-                        if constexpr (PREC == 2 && ORDER == 1)
+                        if constexpr (PREC != 2)
+                            push_one_q<R, DIM, ORDER>(s_hot, s_hot.sp[spi], S, cur, sEBd, fx, s_emax, V, sQw,
+                                                      s_qtail + warp, P, K.dtd, kq, qsd, p, in, sd->err);
+                        else if constexpr (ORDER == 1)
                             push_one_f32lin<DIM>(s_hot, s_hot.sp[spi], cur, sEB, V, sQw, s_qtail + warp, P, K.jf,
                                                  K.dtd, kq, qs, p, in, sd->err);
                         else
-                            push_one<R, DIM, ORDER>(s_hot, s_hot.sp[spi], cur, sEB, sD, V, sQw, s_qtail + warp, P,
+                            push_one<R, DIM, ORDER>(s_hot, s_hot.sp[spi], cur, sEB, V, sQw, s_qtail + warp, P,
                                                     K.jf, K.dtd, kq, qs, p, in, sd->err);
                     };
                     // a full ring (32 queued crossings) is drained by the whole warp
@@ -1533,28 +1967,30 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                             __syncwarp();
                         }
                     };
-                    if constexpr (PREC == 2 && PPT == 1) {
-                        // FP32: the particle loads are the latency the loop waits on; each
+                    if constexpr (PPT == 1) {
+                        // the particle loads are a latency the loop waits on; each
                         // lane stages its next particle into shared memory with cp.async
                         // one iteration ahead (two buffers per warp, the lane's own column)
                         double* const pbw = smem + P.pb_off + warp * (2 * PIN_SLOTS) + lane;
-                        const int64_t pf = s0 + warp * 32 + lane;
-                        if (pf < s1) stage_in<DIM>(s_hot.sp[spi], pf, pbw);
+                        const int64_t pf = first + lane;
+                        if (P.staged && pf < s1) stage_in<DIM>(s_hot.sp[spi], pf, pbw);
                         cp_async_commit();
                         unsigned buf = 0u;
-                        for (int64_t p0 = s0 + warp * 32; p0 < s1; p0 += (int64_t)blockDim.x) {
+                        for (int64_t p0 = first; p0 < s1; p0 += (int64_t)blockDim.x) {
                             const int64_t pn = p0 + blockDim.x + lane;
-                            if (pn < s1) stage_in<DIM>(s_hot.sp[spi], pn, pbw + (buf ^ 1u) * PIN_SLOTS);
+                            if (P.staged && pn < s1) stage_in<DIM>(s_hot.sp[spi], pn, pbw + (buf ^ 1u) * PIN_SLOTS);
                             cp_async_commit();
                             cp_async_wait<1>();
                             const int64_t p = p0 + lane;
-                            if (p < s1) push(p, read_staged<DIM>(pbw + buf * PIN_SLOTS));
+                            if (p < s1)
+                                push(p, P.staged ? read_staged<DIM>(pbw + buf * PIN_SLOTS)
+                                                 : load_one<DIM>(s_hot.sp[spi], p));
                             buf ^= 1u;
                             drain_full();
                         }
                         cp_async_wait<0>();
                     } else {
-                        for (int64_t p0 = s0 + warp * (32 * PPT); p0 < s1; p0 += (int64_t)blockDim.x * PPT) {
+                        for (int64_t p0 = first; p0 < s1; p0 += (int64_t)blockDim.x * PPT) {
                             PIn in[PPT];
 #pragma unroll
                             for (int q = 0; q < PPT; ++q) {
@@ -1572,6 +2008,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     __syncwarp();
                 }
                 if (cap_clk) my_clk += clock64() - c0;
+                if (lane == 0 && cap_time) my_ns += globaltimer() - t0;
             }
         }
         // in-situ cost: thread clocks -> warp sum -> shared -> one global add per unit
@@ -1579,14 +2016,17 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
             unsigned long long ws = warp_sum_u64(my_clk);
             if ((threadIdx.x & 31) == 0 && ws) atomicAdd(&s_cost, ws);
         }
+        if (lane == 0 && my_ns) atomicAdd(&s_time, (unsigned long long)my_ns);
         __syncthreads();
         if (threadIdx.x == 0) {
             if (s_cost) atomicAdd((unsigned long long*)(S.cost_clock + unit.box), s_cost);
             s_cost = 0ull;
-            // kernel-time cost: wall span of the unit on this CTA (ns)
+            // kernel-time cost: span of the unit's particle loops, the mean over the
+            // CTA's warps (a unit that fills them is charged its wall time, one that
+            // leaves warps idle the share it uses)
             if (cap_time)
-                atomicAdd((unsigned long long*)(S.cost_time + unit.box),
-                          (unsigned long long)(globaltimer() - t_unit0));
+                atomicAdd((unsigned long long*)(S.cost_time + unit.box), s_time / (unsigned long long)(blockDim.x >> 5));
+            s_time = 0ull;
         }
     }
     if (cur.t >= 0) drain_ring(sims[cur.sim]);

@@ -12,8 +12,7 @@ size_t pic_particle_smem_bytes(int dim, int order, const int T[3], int threads, 
         ebs[a] = act ? T[a] + (order == 1 ? 2 : order == 2 ? 3 : 4) : 1;
     }
     if (order == 2) ebs[0] += 1;  // even x extent for TMA (16-byte rows)
-    // tiles (the x differences for linear FP64; the particle staging buffers
-    // for the FP32 variant, prec 2) + alignment slack of the dynamic base; the
-    // rings of crossing particles are in global memory
-    return smem_plan(ebs, uses_xdiff(prec, order), prec == 2).bytes + 128;
+    // the tile, the particle staging buffers and the alignment slack of the
+    // dynamic base; the rings of crossing particles are in global memory
+    return smem_plan(ebs).bytes + 128;
 }
