@@ -492,6 +492,7 @@ pic_status configure_launch(pic_sim* s) {
     int resident = pic_particle_occupancy(s->h.dim, s->h.order, s->minb, s->ppt, s->threads, s->smem, s->prec);
     if (resident < 1) return fail(s, PIC_EUNSUPPORTED, "particle kernel does not fit on an SM");
     int per_sm = std::max(1, std::min(s->ctas_per_sm, resident));
+    per_sm = std::max(1, std::min(per_sm, PIC_RING_WARPS_PER_SM / (s->threads / 32)));
     s->ctas = s->nsm * per_sm;
     s->graph_dirty = true;
     return PIC_OK;
@@ -1229,7 +1230,7 @@ pic_status pic_set_launch(pic_sim* s, const pic_launch_cfg* cfg) {
         s->threads = cfg->threads;
     }
     if (cfg->ctas_per_sm > 0) {
-        if (cfg->ctas_per_sm > PIC_RING_CTAS_PER_SM) return fail(s, PIC_EINVAL, "ctas_per_sm must be 1..4");
+        if (cfg->ctas_per_sm > PIC_MAX_CTAS_PER_SM) return fail(s, PIC_EINVAL, "ctas_per_sm must be 1..4");
         s->ctas_per_sm = cfg->ctas_per_sm;
     }
     const int old_split = s->split;

