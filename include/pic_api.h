@@ -154,7 +154,9 @@ enum { PIC_LB_NONE = 0, PIC_LB_STATIC = 1, PIC_LB_DYNAMIC = 2 };
 enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
 
 /* Parameters of the load-balancing routine (Sec. 2.2; scans in Sec. 3.3).
- *   mode        NONE: work in box order, boxes never split, mapping fixed;
+ *   mode        NONE: work in box order, one unit per box, mapping fixed (a
+ *               mapping with at most half as many units as CTAs has each unit
+ *               shared by several CTAs, in every mode);
  *               STATIC: balance once, at the first interval, threshold 0;
  *               DYNAMIC: balance every `interval` steps with threshold theta.
  *   interval    steps between load-balancing calls (Sec. 3.3 scans 1..300).

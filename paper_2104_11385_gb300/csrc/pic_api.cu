@@ -253,9 +253,45 @@ void build_plan(pic_sim* s, const std::vector<pic::Unit>& units, const std::vect
     }
 }
 
+// CTAs that share one work unit.  A mapping with at most half as many units as
+// persistent CTAs (8 boxes on 152 SMs) would leave most of the chip idle, so
+// each unit is then cut into equal parts that different CTAs pull, down to 256
+// particles (one round of a CTA's threads).  The plan itself, its costs and its
+// efficiency stay per unit.  16^3 cells in 8 boxes, 32768 particles, one CTA per
+// SM: the particle kernel takes 40 us against 137.
+int64_t unit_share(const pic_sim* s, int64_t nu) {
+    if (nu == 0 || 2 * nu > s->ctas) return 1;
+    int64_t np = 0;
+    for (int i = 0; i < s->h.nsp; ++i) np += s->np_init[i];
+    return std::max<int64_t>(1, std::min<int64_t>(s->ctas / nu, np / nu / 256));
+}
+
+// Particles below which a heavy box is not cut further.  A unit costs about 14
+// us of scheduling, tile staging and partly filled rounds before any balance is
+// gained (128^3 foil, 8.4 M particles on 304 CTAs: 1.48 ms in units of 1725
+// particles, 1.31 ms in units of 6900), so units hold at least 4096 particles,
+// or a quarter of a worker's share where that is less, and never below 1024.
+int64_t min_unit_particles(const std::vector<int64_t>& np, int n_workers) {
+    int64_t total = 0;
+    for (int64_t n : np) total += n;
+    return std::max<int64_t>(1024, std::min<int64_t>(4096, total / (4 * std::max(1, n_workers))));
+}
+
 pic_status upload_plan(pic_sim* s) {
-    SimPlan& P = s->plan;
-    int64_t nu = (int64_t)P.units.size();
+    const SimPlan& P = s->plan;
+    std::vector<UnitDev> units = P.units;
+    std::vector<int32_t> list_off = P.list_off;
+    int nlists = P.nlists;
+    const int64_t share = unit_share(s, (int64_t)units.size());
+    if (share > 1) {
+        units.clear();
+        for (const UnitDev& u : P.units)
+            for (int32_t k = 0; k < (int32_t)share; ++k)
+                units.push_back(UnitDev{u.sim, u.box, (int32_t)(u.chunk * share + k), (int32_t)(u.nchunks * share)});
+        nlists = 1;
+        list_off = {0, (int32_t)units.size()};
+    }
+    const int64_t nu = (int64_t)units.size();
     if (nu > s->units_cap) {
         int64_t cap = std::max<int64_t>(nu, 2 * s->units_cap);
         UnitDev* nu_ptr = nullptr;
@@ -264,13 +300,13 @@ pic_status upload_plan(pic_sim* s) {
         s->units_cap = cap;
         CU(s, cudaMemcpyAsync(s->ds, &s->hs, sizeof(SchedDev), cudaMemcpyHostToDevice, s->stream));
     }
-    if (P.nlists + 1 > 8192) return fail(s, PIC_EINVAL, "too many work lists (%d)", P.nlists);
+    if (nlists + 1 > 8192) return fail(s, PIC_EINVAL, "too many work lists (%d)", nlists);
     if (nu > 0)
-        CU(s, cudaMemcpyAsync(s->hs.units, P.units.data(), nu * sizeof(UnitDev),
+        CU(s, cudaMemcpyAsync(s->hs.units, units.data(), nu * sizeof(UnitDev),
                               cudaMemcpyHostToDevice, s->stream));
-    CU(s, cudaMemcpyAsync(s->hs.list_off, P.list_off.data(), P.list_off.size() * sizeof(int32_t),
+    CU(s, cudaMemcpyAsync(s->hs.list_off, list_off.data(), list_off.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice, s->stream));
-    int32_t meta[2] = {P.nlists, 0};
+    int32_t meta[2] = {nlists, 0};
     CU(s, cudaMemcpyAsync(s->hs.meta, meta, sizeof meta, cudaMemcpyHostToDevice, s->stream));
     CU(s, cudaStreamSynchronize(s->stream));
     return PIC_OK;
@@ -410,7 +446,7 @@ pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_re
     const double e_old = plan_efficiency(s, costs);
     const int split = p.split > 0 ? p.split : s->split;
     std::vector<pic::Unit> units =
-        pic::make_units(costs.data(), np.data(), nb, nw, split, 256, true);
+        pic::make_units(costs.data(), np.data(), nb, nw, split, min_unit_particles(np, nw), true);
     std::vector<double> uc;
     std::vector<int32_t> assign;
     map_units(s, p, units, nw, uc, assign);
@@ -580,7 +616,7 @@ pic_status replan(pic_sim* s) {
     const int nw = n_workers_for(s, p);
     const int split = p.split > 0 ? p.split : s->split;
     std::vector<pic::Unit> units = pic::make_units(s->last_costs.data(), s->last_np.data(),
-                                                   s->h.nboxes, nw, split, 256, true);
+                                                   s->h.nboxes, nw, split, min_unit_particles(s->last_np, nw), true);
     std::vector<double> uc;
     std::vector<int32_t> assign;
     map_units(s, p, units, nw, uc, assign);  // the simulation's own policy

@@ -95,3 +95,18 @@ def test_tile_without_staging_buffers(order):
     sim.step(4)
     ref.step(4)
     compare(sim, ref, wl)
+
+
+@pytest.mark.parametrize("mode", ["none", "queue", "lists"])
+@pytest.mark.parametrize("npart", [1, 700, 40000])
+def test_few_boxes_shared_by_many_ctas(mode, npart):
+    wl = workloads.random_plasma(72, 3, (16, 16, 8), (8, 8, 8), (0.3, 0.3, 0.3), 1, nspecies=2, npart=npart, umax=1.0)
+    sim, ref = make_gpu(wl), make_oracle(wl)
+    if mode != "none":
+        sim.set_lb_params(mode=pic.LB_DYNAMIC, interval=2, theta=0.0, cost=pic.COST_HEURISTIC,
+                          sched=pic.SCHED_QUEUE if mode == "queue" else pic.SCHED_LISTS)
+    sim.step(5)
+    ref.step(5)
+    compare(sim, ref, wl)
+    _, counts = sim.box_costs(pic.COST_HEURISTIC)
+    assert np.array_equal(counts, ref.box_counts(wl["box"]))
