@@ -485,15 +485,17 @@ pic_status enqueue_step(pic_sim* s, bool with_events) {
     if (with_events) CU(s, cudaEventRecord(s->ev[1], s->stream));
     CU(s, pic_launch_fields(s->d, h, s->stream));
     if (with_events) CU(s, cudaEventRecord(s->ev[2], s->stream));
-    for (int sp = 0; sp < h.nsp; ++sp) CU(s, pic_launch_sort(s->d, h, sp, s->stream));
-    CU(s, pic_launch_finish(s->d, s->ds, s->stream));
+    CU(s, pic_launch_sort_all(s->d, h, s->stream));
+    CU(s, pic_launch_finish(s->d, s->ds, true, s->stream));
     if (with_events) CU(s, cudaEventRecord(s->ev[3], s->stream));
     return PIC_OK;
 }
 
 int count_kernels(const pic_sim* s) {
-    int k = (s->h.nsp > 0 ? 1 : 0) + 1 + 3 + (s->h.absorb > 0 ? 1 : 0) + 1 + 3 * s->h.nsp + 1;
-    return k;
+    const SimDev& h = s->h;
+    const bool multi = (int64_t)h.ntiles + 1 > 8192;
+    const int sort = h.nsp > 0 ? (multi ? 3 * h.nsp : 1) + 1 : 0;
+    return (h.nsp > 0 ? 1 : 0) + 3 + (h.absorb > 0 ? 1 : 0) + 1 + sort + 1;
 }
 
 pic_status capture_graph(pic_sim* s) {

@@ -25,14 +25,15 @@ __device__ __forceinline__ const SimDev& slot_sim(const SimDev* sims, const int*
 // lanes along x (coalesced): f(i, j, k, o, oi, oj, ok) gets the cell's padded
 // index o and those of its periodic neighbours along x, y and z, the next ones
 // (FWD) or the previous ones.  Only the row index is divided.
+// blk of nblk: the block's place among those that share the rows
 template <int DIM, bool FWD, class F>
-__device__ __forceinline__ void for_cells_by_row(const SimDev& S, F&& f) {
+__device__ __forceinline__ void for_cells_by_row(const SimDev& S, int blk, int nblk, F&& f) {
     const int nx = S.n[0], ny = S.n[1], nz = S.n[2];
     const bool all_owned = S.owner == nullptr;
     const int wpb = blockDim.x >> 5;
     const int64_t rows = (int64_t)ny * nz;
     auto nb = [](int i, int n) { return FWD ? nxt(i, n) : prv(i, n); };
-    for (int64_t r = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += (int64_t)gridDim.x * wpb) {
+    for (int64_t r = (int64_t)blk * wpb + (threadIdx.x >> 5); r < rows; r += (int64_t)nblk * wpb) {
         const int k = (int)(r / ny), j = (int)(r - (int64_t)k * ny);
         const int64_t row = pidx(S, 0, j, k);
         const int64_t dj = (DIM == 3) ? pidx(S, 0, nb(j, ny), k) - row : 0;
@@ -46,9 +47,78 @@ __device__ __forceinline__ void for_cells_by_row(const SimDev& S, F&& f) {
     }
 }
 
+// Visits the guard cells of the padded arrays, one warp per padded row (b, e):
+// the whole row when it lies in a y or z guard layer, else only the x guards
+// at its two ends (at most 8 cells).  f(c, i, j, k) gets the padded index and
+// the interior coordinates of the cell (outside [0, n) along some axis).  The
+// guards are a few per cent of the padded volume, and no thread divides
+// anything but its row index.
+template <class F>
+__device__ __forceinline__ void for_guard_cells(const SimDev& S, int blk, int nblk, F&& f) {
+    const int px = S.pn[0], py = S.pn[1], pz = S.pn[2];
+    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+    const int gl = S.g[0], gx = px - S.n[0];  // left x guards, both x guards
+    const int64_t rows = (int64_t)py * pz;
+    for (int64_t r = (int64_t)blk * wpb + (threadIdx.x >> 5); r < rows; r += (int64_t)nblk * wpb) {
+        const int e = (int)(r / py), b = (int)(r - (int64_t)e * py);
+        const int j = b - S.g[1], k = e - S.g[2];
+        const int64_t row0 = r * px;
+        if (j < 0 || j >= S.n[1] || k < 0 || k >= S.n[2]) {
+            for (int a = lane; a < px; a += 32) f(row0 + a, a - gl, j, k);
+        } else if (lane < gx) {
+            const int a = lane < gl ? lane : S.n[0] + lane;
+            f(row0 + a, a - gl, j, k);
+        }
+    }
+}
+
+__device__ __forceinline__ int wrap_cell(int i, int n) {
+    const int r = i % n;
+    return r < 0 ? r + n : r;
+}
+
+// Current deposited in the guard cells of the padded J arrays (the particle
+// kernel's reductions reach up to 2 cells below and 3 above the domain) added
+// to its periodic image inside the domain.  Several guard cells share an image
+// (edges, corners), hence the reductions; guard cells holding zero are skipped.
+__device__ __forceinline__ void fold_j(const SimDev& S, int blk, int nblk) {
+    for_guard_cells(S, blk, nblk, [&](int64_t c, int i, int j, int k) {
+        const int64_t dst = pidx(S, wrap_cell(i, S.n[0]), wrap_cell(j, S.n[1]), wrap_cell(k, S.n[2]));
+#pragma unroll
+        for (int comp = 6; comp < 9; ++comp) {
+            const double v = S.F[comp][c];
+            if (v != 0.0) atomicAdd(S.F[comp] + dst, v);
+        }
+    });
+}
+__global__ void fold_j_kernel(const SimDev* __restrict__ sims, const int* __restrict__ slots) {
+    fold_j(slot_sim(sims, slots), blockIdx.x, gridDim.x);
+}
+
+// the antenna's time factor of the step under way
+__device__ __noinline__ double antenna_amp(const SimDev& S) {
+    const LaserDev& L = S.las;
+    const double t = ((double)(*S.step) + 0.5) * S.dt;
+    const double tt = (t - L.t_peak) / L.tau;
+    return 2.0 * L.a0 / S.d[2] * exp(-tt * tt) * sin(L.omega * (t - L.t_peak));
+}
+
+// B half step.  A step's first one also folds the current (nfold further
+// blocks: the two touch different arrays, and share one launch) and leaves the
+// antenna's time factor for the E step (in one thread: FP64 exp and sin are
+// over a hundred FP64 instructions at 1/64 of the FP32 rate; computed by every
+// block of the E step, with a launch more for the fold, the field phase of the
+// 128^3 foil took 289 us against 255).
 template <int DIM>
-__global__ void b_half_kernel(const SimDev* __restrict__ sims, const int* __restrict__ slots) {
+__global__ void b_half_kernel(const SimDev* __restrict__ sims, const int* __restrict__ slots, int first, int nfold) {
     const SimDev& S = slot_sim(sims, slots);
+    const int nb = gridDim.x - nfold;
+    if ((int)blockIdx.x >= nb) {
+        fold_j(S, blockIdx.x - nb, nfold);
+        return;
+    }
+    // (read by later launches only)
+    if (first && blockIdx.x == 0 && threadIdx.x == 0 && S.las.on) const_cast<SimDev&>(S).las.amp = antenna_amp(S);
     // B -= (dt/2) curl E with dt/(2 dx) folded into the differences: two FMAs
     // per component
     const double h = 0.5 * S.dt;
@@ -59,7 +129,7 @@ __global__ void b_half_kernel(const SimDev* __restrict__ sims, const int* __rest
     double* __restrict__ Bx = S.F[3];
     double* __restrict__ By = S.F[4];
     double* __restrict__ Bz = S.F[5];
-    for_cells_by_row<DIM, true>(S, [&](int, int, int, int64_t o, int64_t oi, int64_t oj, int64_t ok) {
+    for_cells_by_row<DIM, true>(S, blockIdx.x, nb, [&](int, int, int, int64_t o, int64_t oi, int64_t oj, int64_t ok) {
         const double ez = Ez[o], ey = Ey[o], ex = Ex[o];
         Bx[o] = fma(Ey[ok] - ey, hz, fma(-(Ez[oj] - ez), hy, Bx[o]));
         By[o] = fma(Ez[oi] - ez, hx, fma(-(Ex[ok] - ex), hz, By[o]));
@@ -94,21 +164,8 @@ __global__ void e_kernel(const SimDev* __restrict__ sims, const int* __restrict_
     const double* __restrict__ Jy = S.F[7];
     const double* __restrict__ Jz = S.F[8];
     const LaserDev L = S.las;
-    // the antenna's time factor, once per block (FP64 exp and sin are dozens
-    // of FP64 instructions, at 1/64 of the FP32 rate)
-    __shared__ double s_amp;
-    if (threadIdx.x == 0) {
-        double a = 0.0;
-        if (L.on) {
-            double t = ((double)(*S.step) + 0.5) * dt;
-            double tt = (t - L.t_peak) / L.tau;
-            a = 2.0 * L.a0 / S.d[2] * exp(-tt * tt) * sin(L.omega * (t - L.t_peak));
-        }
-        s_amp = a;
-    }
-    __syncthreads();
-    const double amp = s_amp;
-    for_cells_by_row<DIM, false>(S, [&](int i, int j, int k, int64_t o, int64_t oi, int64_t oj, int64_t ok) {
+    const double amp = L.amp;
+    for_cells_by_row<DIM, false>(S, blockIdx.x, gridDim.x, [&](int i, int j, int k, int64_t o, int64_t oi, int64_t oj, int64_t ok) {
         const double bx = Bx[o], by = By[o], bz = Bz[o];
         double jx = Jx[o];
         if (L.on && k == L.k_ant) {
@@ -145,57 +202,11 @@ __global__ void damp_kernel(const SimDev* __restrict__ sims, const int* __restri
     }
 }
 
-// Visits the guard cells of the padded arrays, one warp per padded row (b, e):
-// the whole row when it lies in a y or z guard layer, else only the x guards
-// at its two ends (at most 8 cells).  f(c, i, j, k) gets the padded index and
-// the interior coordinates of the cell (outside [0, n) along some axis).  The
-// guards are a few per cent of the padded volume, and no thread divides
-// anything but its row index.
-template <class F>
-__device__ __forceinline__ void for_guard_cells(const SimDev& S, F&& f) {
-    const int px = S.pn[0], py = S.pn[1], pz = S.pn[2];
-    const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-    const int gl = S.g[0], gx = px - S.n[0];  // left x guards, both x guards
-    const int64_t rows = (int64_t)py * pz;
-    for (int64_t r = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); r < rows; r += (int64_t)gridDim.x * wpb) {
-        const int e = (int)(r / py), b = (int)(r - (int64_t)e * py);
-        const int j = b - S.g[1], k = e - S.g[2];
-        const int64_t row0 = r * px;
-        if (j < 0 || j >= S.n[1] || k < 0 || k >= S.n[2]) {
-            for (int a = lane; a < px; a += 32) f(row0 + a, a - gl, j, k);
-        } else if (lane < gx) {
-            const int a = lane < gl ? lane : S.n[0] + lane;
-            f(row0 + a, a - gl, j, k);
-        }
-    }
-}
-
-__device__ __forceinline__ int wrap_cell(int i, int n) {
-    const int r = i % n;
-    return r < 0 ? r + n : r;
-}
-
-// Current deposited in the guard cells of the padded J arrays (the particle
-// kernel's reductions reach up to 2 cells below and 3 above the domain) added
-// to its periodic image inside the domain.  Several guard cells share an image
-// (edges, corners), hence the reductions; guard cells holding zero are skipped.
-__global__ void fold_j_kernel(const SimDev* __restrict__ sims, const int* __restrict__ slots) {
-    const SimDev& S = slot_sim(sims, slots);
-    for_guard_cells(S, [&](int64_t c, int i, int j, int k) {
-        const int64_t dst = pidx(S, wrap_cell(i, S.n[0]), wrap_cell(j, S.n[1]), wrap_cell(k, S.n[2]));
-#pragma unroll
-        for (int comp = 6; comp < 9; ++comp) {
-            const double v = S.F[comp][c];
-            if (v != 0.0) atomicAdd(S.F[comp] + dst, v);
-        }
-    });
-}
-
 // periodic images into the guard cells of components [c0, c0+nc)
 __global__ void guard_kernel(const SimDev* __restrict__ sims, const int* __restrict__ slots, int c0,
                              int nc) {
     const SimDev& S = slot_sim(sims, slots);
-    for_guard_cells(S, [&](int64_t c, int i, int j, int k) {
+    for_guard_cells(S, blockIdx.x, gridDim.x, [&](int64_t c, int i, int j, int k) {
         const int64_t src = pidx(S, wrap_cell(i, S.n[0]), wrap_cell(j, S.n[1]), wrap_cell(k, S.n[2]));
         for (int comp = c0; comp < c0 + nc; ++comp) S.F[comp][c] = S.F[comp][src];
     });
@@ -299,20 +310,21 @@ int blocks_for(int64_t n, int t) {
     return (int)b;
 }
 
+// blocks of the row kernels: 8 rows each
+int row_blocks(const SimDev& h) { return blocks_for((int64_t)h.n[1] * h.n[2] * 32, 256); }
+
 }  // namespace
 
 cudaError_t pic_launch_fields(const SimDev* dsim, const SimDev& h, cudaStream_t st) {
-    const int64_t ncell = (int64_t)h.n[0] * h.n[1] * h.n[2];
-    const int nb = blocks_for(ncell, 256);
-    fold_j_kernel<<<blocks_for(guard_rows(h) * 32, 256), 256, 0, st>>>(dsim, nullptr);
+    const int nb = row_blocks(h), nf = blocks_for(guard_rows(h) * 32, 256);
     if (h.dim == 3) {
-        b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr);
+        b_half_kernel<3><<<nb + nf, 256, 0, st>>>(dsim, nullptr, 1, nf);
         e_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr);
-        b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr);
+        b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr, 0, 0);
     } else {
-        b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr);
+        b_half_kernel<2><<<nb + nf, 256, 0, st>>>(dsim, nullptr, 1, nf);
         e_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr);
-        b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr);
+        b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr, 0, 0);
     }
     if (h.absorb > 0) {
         int64_t t = (int64_t)h.n[0] * h.n[1] * 2 * h.absorb;
@@ -327,11 +339,10 @@ cudaError_t pic_launch_fold(const SimDev* dsim, const SimDev& h, cudaStream_t st
 }
 
 cudaError_t pic_launch_field_stage(const SimDev* dsim, const SimDev& h, int stage, cudaStream_t st) {
-    const int64_t ncell = (int64_t)h.n[0] * h.n[1] * h.n[2];
-    const int nb = blocks_for(ncell, 256);
+    const int nb = row_blocks(h);
     if (stage == 0 || stage == 2) {
-        if (h.dim == 3) b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr);
-        else b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr);
+        if (h.dim == 3) b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr, stage == 0, 0);
+        else b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr, stage == 0, 0);
         if (stage == 2 && h.absorb > 0) {
             int64_t t = (int64_t)h.n[0] * h.n[1] * 2 * h.absorb;
             damp_kernel<<<blocks_for(t, 256), 256, 0, st>>>(dsim, nullptr);
@@ -356,15 +367,16 @@ cudaError_t pic_launch_fields_multi(const SimDev* sims, const int* slots, int ns
                                     cudaStream_t st) {
     if (nslots <= 0) return cudaSuccess;
     const dim3 g(blocks_for(max_cells, 256) / 4 + 1, nslots);
-    fold_j_kernel<<<dim3(blocks_for(max_padded, 256) / 4 + 1, nslots), 256, 0, st>>>(sims, slots);
+    const int nf = blocks_for(max_padded, 256) / 4 + 1;
+    const dim3 g1(g.x + nf, nslots);
     if (dim == 3) {
-        b_half_kernel<3><<<g, 256, 0, st>>>(sims, slots);
+        b_half_kernel<3><<<g1, 256, 0, st>>>(sims, slots, 1, nf);
         e_kernel<3><<<g, 256, 0, st>>>(sims, slots);
-        b_half_kernel<3><<<g, 256, 0, st>>>(sims, slots);
+        b_half_kernel<3><<<g, 256, 0, st>>>(sims, slots, 0, 0);
     } else {
-        b_half_kernel<2><<<g, 256, 0, st>>>(sims, slots);
+        b_half_kernel<2><<<g1, 256, 0, st>>>(sims, slots, 1, nf);
         e_kernel<2><<<g, 256, 0, st>>>(sims, slots);
-        b_half_kernel<2><<<g, 256, 0, st>>>(sims, slots);
+        b_half_kernel<2><<<g, 256, 0, st>>>(sims, slots, 0, 0);
     }
     if (any_absorb) damp_kernel<<<g, 256, 0, st>>>(sims, slots);
     const dim3 gp(blocks_for(max_padded, 256) / 4 + 1, nslots);

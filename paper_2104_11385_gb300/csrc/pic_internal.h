@@ -57,6 +57,7 @@ struct LaserDev {
     int on;
     int k_ant;
     double a0, w0, tau, t_peak, omega, xc, yc;
+    double amp;  // time factor of the step under way, written by its first field kernel
 };
 
 struct SimDev {
@@ -166,9 +167,11 @@ cudaError_t pic_launch_particles(int dim, int order, const LaunchCfg& cfg, size_
                                  const SchedDev* sched, SimDev* sims, cudaStream_t st);
 cudaError_t pic_launch_fields(const SimDev* dsim, const SimDev& hsim, cudaStream_t st);
 cudaError_t pic_launch_sort(const SimDev* dsim, const SimDev& hsim, int sp, cudaStream_t st);
+cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, cudaStream_t st);
 cudaError_t pic_launch_initial_keys(const SimDev* dsim, const SimDev& hsim, int sp,
                                     int64_t np, cudaStream_t st);
-cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, cudaStream_t st);
+// swap: exchange every species' buffers (after pic_launch_sort_all)
+cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, bool swap, cudaStream_t st);
 cudaError_t pic_launch_box_counts(const SimDev* dsim, const SimDev& hsim, int64_t* out,
                                   cudaStream_t st);
 cudaError_t pic_launch_rho(const SimDev* dsim, const SimDev& hsim, double* rho, double rho0,

@@ -179,11 +179,7 @@ __global__ void pic_scatter_kernel(SimDev* __restrict__ sims, const int* __restr
     }
 }
 
-__global__ void pic_swap_kernel(SimDev* __restrict__ sims, const int* __restrict__ slots, int sp_idx) {
-    SimDev& S = sims[slots ? slots[blockIdx.y] : 0];
-    if (sp_idx < 0) sp_idx = blockIdx.x;
-    if (sp_idx >= S.nsp || threadIdx.x != 0) return;
-    SpeciesDev& sp = S.sp[sp_idx];
+__device__ __forceinline__ void swap_buffers(SpeciesDev& sp) {
     for (int a = 0; a < 7; ++a) {
         double* t = sp.cur[a];
         sp.cur[a] = sp.alt[a];
@@ -194,13 +190,21 @@ __global__ void pic_swap_kernel(SimDev* __restrict__ sims, const int* __restrict
     sp.id_alt = ti;
 }
 
+__global__ void pic_swap_kernel(SimDev* __restrict__ sims, int sp_idx) {
+    if (threadIdx.x == 0) swap_buffers(sims[0].sp[sp_idx]);
+}
+
+// end of a step: list heads and step counter, and (swap) the buffers of every
+// species that the step's scatter filled
 __global__ void pic_finish_kernel(SimDev* __restrict__ sims, const int* __restrict__ slots,
-                                  const SchedDev* __restrict__ sd) {
+                                  const SchedDev* __restrict__ sd, int swap) {
+    SimDev& S = sims[slots ? slots[blockIdx.y] : 0];
     if (blockIdx.y == 0) {
         const int nlists = sd->meta[0];
         for (int i = threadIdx.x; i < nlists; i += blockDim.x) sd->head[i] = 0;
     }
-    if (threadIdx.x == 0) *sims[slots ? slots[blockIdx.y] : 0].step += 1;
+    if (threadIdx.x == 0) *S.step += 1;
+    if (swap && (int)threadIdx.x < S.nsp) swap_buffers(S.sp[threadIdx.x]);
 }
 
 template <int DIM>
@@ -335,7 +339,33 @@ cudaError_t pic_launch_sort(const SimDev* dsim, const SimDev& hsim, int sp, cuda
     int64_t cap = hsim.sp[sp].cap;
     if (hsim.dim == 3) pic_scatter_kernel<3><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
     else pic_scatter_kernel<2><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
-    pic_swap_kernel<<<1, 32, 0, st>>>(d, nullptr, sp);
+    pic_swap_kernel<<<1, 32, 0, st>>>(d, sp);
+    return cudaGetLastError();
+}
+
+// the sort of a step: every species in the same two launches (three more per
+// species for large tile counts); the swap of their buffers is left to
+// pic_finish_kernel.  Against three launches per species this takes one launch
+// (one species) to four (two) off a step, about 2 us each where launches count.
+cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, cudaStream_t st) {
+    if (hsim.nsp == 0) return cudaSuccess;
+    SimDev* d = const_cast<SimDev*>(dsim);
+    const int64_t N = (int64_t)hsim.ntiles + 1;
+    const int64_t nparts = (N + kScanBlock - 1) / kScanBlock;
+    if (N > 8 * kScanBlock && hsim.scan_part && nparts <= hsim.scan_part_cap) {
+        for (int sp = 0; sp < hsim.nsp; ++sp) {
+            pic_scan_part_kernel<<<(int)nparts, kScanBlock, 0, st>>>(d, sp);
+            pic_scan_top_kernel<<<1, kScanBlock, 0, st>>>(d, sp, (int)nparts);
+            pic_scan_final_kernel<<<(int)nparts, kScanBlock, 0, st>>>(d, sp);
+        }
+    } else {
+        pic_scan_kernel<<<hsim.nsp, 1024, 0, st>>>(d, nullptr, -1);
+    }
+    int64_t cap = 1;
+    for (int sp = 0; sp < hsim.nsp; ++sp) cap = std::max(cap, hsim.sp[sp].cap);
+    const dim3 g(grid_for(cap, 256), 1, hsim.nsp);
+    if (hsim.dim == 3) pic_scatter_kernel<3><<<g, 256, 0, st>>>(d, nullptr, -1);
+    else pic_scatter_kernel<2><<<g, 256, 0, st>>>(d, nullptr, -1);
     return cudaGetLastError();
 }
 
@@ -346,14 +376,13 @@ cudaError_t pic_launch_sort_multi(SimDev* sims, const int* slots, int nslots, in
     const dim3 g(grid_for(max_cap, 256) / 4 + 1, nslots, PIC_MAXSP);
     if (dim == 3) pic_scatter_kernel<3><<<g, 256, 0, st>>>(sims, slots, -1);
     else pic_scatter_kernel<2><<<g, 256, 0, st>>>(sims, slots, -1);
-    pic_swap_kernel<<<dim3(PIC_MAXSP, nslots), 32, 0, st>>>(sims, slots, -1);
     return cudaGetLastError();
 }
 
 cudaError_t pic_launch_finish_multi(SimDev* sims, const int* slots, int nslots, const SchedDev* sched,
                                     cudaStream_t st) {
     if (nslots <= 0) return cudaSuccess;
-    pic_finish_kernel<<<dim3(1, nslots), 256, 0, st>>>(sims, slots, sched);
+    pic_finish_kernel<<<dim3(1, nslots), 256, 0, st>>>(sims, slots, sched, 1);
     return cudaGetLastError();
 }
 
@@ -377,8 +406,8 @@ cudaError_t pic_launch_keys_range(const SimDev* dsim, const SimDev& hsim, int sp
     return cudaGetLastError();
 }
 
-cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, cudaStream_t st) {
-    pic_finish_kernel<<<1, 256, 0, st>>>(dsim, nullptr, sched);
+cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, bool swap, cudaStream_t st) {
+    pic_finish_kernel<<<1, 256, 0, st>>>(dsim, nullptr, sched, swap ? 1 : 0);
     return cudaGetLastError();
 }
 
