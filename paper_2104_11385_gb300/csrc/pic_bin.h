@@ -11,7 +11,7 @@
 struct BinGeom {
     int dim;
     int n[3], bsz[3], nb[3];
-    double d[3];
+    double d[3], inv[3];  // cell sizes and their reciprocals
     int nboxes;
 };
 

@@ -110,3 +110,25 @@ def test_few_boxes_shared_by_many_ctas(mode, npart):
     compare(sim, ref, wl)
     _, counts = sim.box_costs(pic.COST_HEURISTIC)
     assert np.array_equal(counts, ref.box_counts(wl["box"]))
+
+
+@pytest.mark.parametrize("d", [0.25, 0.3, 1.0 / 3.0, 7.0, 1e-3])
+def test_bin_positions_at_cell_faces(d):
+    """k d and its neighbours, also outside the domain: the boxes of the rounded division"""
+    import torch
+    from paper_2104_11385_gb300 import sim as S
+    n, box = (60, 1, 4096), (3, 1, 512)
+    k = np.arange(-4200, 4300, dtype=np.float64)
+    x = np.concatenate([k * d, np.nextafter(k * d, -np.inf), np.nextafter(k * d, np.inf), [0.0, -0.0, 1e-300, -1e-300],
+                        np.random.default_rng(3).uniform(-1, 2, 5000) * n[2] * d])
+    z = x[::-1].copy()
+    off_r, perm_r = orc.bin_particles(2, n, (d, 1.0, d), box, x, np.zeros_like(x), z)
+    off = torch.empty(len(off_r), dtype=torch.int64, device="cuda")
+    perm = torch.empty(x.size, dtype=torch.int64, device="cuda")
+    S.bin_particles(2, n, box, (d, 1.0, d), torch.as_tensor(x, device="cuda"), None, torch.as_tensor(z, device="cuda"),
+                    off, perm)
+    torch.cuda.synchronize()
+    off_g, perm_g = off.cpu().numpy(), perm.cpu().numpy()
+    assert np.array_equal(off_g, off_r)
+    for b in range(len(off_r) - 1):
+        assert np.array_equal(np.sort(perm_g[off_r[b]:off_r[b + 1]]), np.sort(perm_r[off_r[b]:off_r[b + 1]]))
