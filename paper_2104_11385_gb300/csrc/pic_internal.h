@@ -43,6 +43,9 @@ struct SpeciesDev {
     double qw_scale;      // q / (dV dt)-style deposit prefactor (per simulation dims)
     double* cur[7];       // X Y Z ux uy uz w  (current, tile-sorted)
     double* alt[7];       // scatter target
+    // 1: between the steps of one pic_step call the particles stay where the push
+    // left them (cur, not sorted) and id_alt holds, by sorted place, where each is
+    int32_t indirect;
     int64_t* id;
     int64_t* id_alt;
     int32_t* key;         // [cap]
@@ -167,11 +170,12 @@ cudaError_t pic_launch_particles(int dim, int order, const LaunchCfg& cfg, size_
                                  const SchedDev* sched, SimDev* sims, cudaStream_t st);
 cudaError_t pic_launch_fields(const SimDev* dsim, const SimDev& hsim, cudaStream_t st);
 cudaError_t pic_launch_sort(const SimDev* dsim, const SimDev& hsim, int sp, cudaStream_t st);
-cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, cudaStream_t st);
+cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, bool index, cudaStream_t st);
 cudaError_t pic_launch_initial_keys(const SimDev* dsim, const SimDev& hsim, int sp,
                                     int64_t np, cudaStream_t st);
-// swap: exchange every species' buffers (after pic_launch_sort_all)
-cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, bool swap, cudaStream_t st);
+// sort: what pic_launch_sort_all did before it (PIC_SORT_*)
+enum { PIC_SORT_NONE = 0, PIC_SORT_FULL = 1, PIC_SORT_INDEX = 2 };
+cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, int sort, cudaStream_t st);
 cudaError_t pic_launch_box_counts(const SimDev* dsim, const SimDev& hsim, int64_t* out,
                                   cudaStream_t st);
 cudaError_t pic_launch_rho(const SimDev* dsim, const SimDev& hsim, double* rho, double rho0,

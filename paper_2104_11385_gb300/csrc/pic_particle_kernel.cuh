@@ -506,7 +506,12 @@ __device__ __forceinline__ void warp_hist_add(int32_t* count, int key) {
 // would be fetched again for every particle (the loop's stores to the particle
 // arrays might alias them as far as the compiler can tell).
 struct HotSp {
-    double* cur[7];
+    double* src[7];        // read at the particle's place,
+    double* dst[7];        // written at its sorted place (the same, unless indirect)
+    const int64_t* order;  // where the particle of each sorted place is (nullptr: there)
+    const int64_t* id_src;
+    int64_t* id_dst;
+    int64_t cap;
     int32_t* key;
     int32_t* count;
     const int64_t* off;
@@ -544,7 +549,15 @@ __device__ __forceinline__ void stage_hot(HotSim& h, const SimDev& S) {
         h.nsp = S.nsp;
         h.je = exp_range(S.jfac[0], S.dim == 2 ? S.jyfac2d : S.jfac[1], S.jfac[2]);
     } else if (i < S.nsp) {
-        for (int k = 0; k < 7; ++k) h.sp[i].cur[k] = S.sp[i].cur[k];
+        const bool ind = S.sp[i].indirect != 0;
+        for (int k = 0; k < 7; ++k) {
+            h.sp[i].src[k] = S.sp[i].cur[k];
+            h.sp[i].dst[k] = ind ? S.sp[i].alt[k] : S.sp[i].cur[k];
+        }
+        h.sp[i].order = ind ? S.sp[i].id_alt : nullptr;
+        h.sp[i].id_src = S.sp[i].id;
+        h.sp[i].cap = S.sp[i].cap;
+        h.sp[i].id_dst = S.sp[i].id_alt;
         h.sp[i].key = S.sp[i].key;
         h.sp[i].count = S.sp[i].count;
         h.sp[i].off = S.sp[i].off;
@@ -1247,13 +1260,13 @@ struct PIn {
 template <int DIM, class SPV>
 __device__ __forceinline__ PIn load_one(const SPV& sp, int64_t p) {
     PIn in;
-    in.X = sp.cur[0][p];
-    in.Y = (DIM == 3) ? sp.cur[1][p] : 0.0;
-    in.Z = sp.cur[2][p];
-    in.u0 = sp.cur[3][p];
-    in.u1 = sp.cur[4][p];
-    in.u2 = sp.cur[5][p];
-    in.w = sp.cur[6][p];
+    in.X = sp.src[0][p];
+    in.Y = (DIM == 3) ? sp.src[1][p] : 0.0;
+    in.Z = sp.src[2][p];
+    in.u0 = sp.src[3][p];
+    in.u1 = sp.src[4][p];
+    in.u2 = sp.src[5][p];
+    in.w = sp.src[6][p];
     return in;
 }
 
@@ -1263,7 +1276,7 @@ template <int DIM, class SPV>
 __device__ __forceinline__ void stage_in(const SPV& sp, int64_t p, double* slot) {
 #pragma unroll
     for (int a = 0; a < 7; ++a)
-        if (DIM == 3 || a != 1) cp_async_8(slot + 32 * a, sp.cur[a] + p);
+        if (DIM == 3 || a != 1) cp_async_8(slot + 32 * a, sp.src[a] + p);
 }
 template <int DIM>
 __device__ __forceinline__ PIn read_staged(const double* slot) {
@@ -1408,12 +1421,12 @@ __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const Sim
         for (int a = 0; a < 3; ++a) g[a] = DIM == 3 || a != 1 ? min(max(ifloor(x1[a]), 0), S.n[a] - 1) : 0;
         key = tile_key(S, g[0], g[1], g[2]);
     }
-    sp.cur[0][p] = x1[0];
-    if (DIM == 3) sp.cur[1][p] = x1[1];
-    sp.cur[2][p] = x1[2];
-    sp.cur[3][p] = A::to(n0);
-    sp.cur[4][p] = A::to(n1);
-    sp.cur[5][p] = A::to(n2);
+    sp.dst[0][p] = x1[0];
+    if (DIM == 3) sp.dst[1][p] = x1[1];
+    sp.dst[2][p] = x1[2];
+    sp.dst[3][p] = A::to(n0);
+    sp.dst[4][p] = A::to(n1);
+    sp.dst[5][p] = A::to(n2);
     sp.key[p] = key;
     warp_hist_add(sp.count, key);
 }
@@ -1534,12 +1547,12 @@ __device__ __forceinline__ void push_one(const SV& S, const SPV& sp, const Tile&
         if (DIM == 3) own = own && (unsigned)(iy - tl.o[1]) < (unsigned)S.T[1];
         key = own ? tl.t : tile_key(S, ix, iy, iz);
     }
-    sp.cur[0][p] = X;
-    if (DIM == 3) sp.cur[1][p] = Y;
-    sp.cur[2][p] = Z;
-    sp.cur[3][p] = A::to(n0);
-    sp.cur[4][p] = A::to(n1);
-    sp.cur[5][p] = A::to(n2);
+    sp.dst[0][p] = X;
+    if (DIM == 3) sp.dst[1][p] = Y;
+    sp.dst[2][p] = Z;
+    sp.dst[3][p] = A::to(n0);
+    sp.dst[4][p] = A::to(n1);
+    sp.dst[5][p] = A::to(n2);
     sp.key[p] = key;
     warp_hist_add(sp.count, key);
 }
@@ -1728,12 +1741,12 @@ __device__ __forceinline__ void push_one_f32lin(const SV& S, const SPV& sp, cons
             key = tile_key(S, min(max(g[0], 0), S.n[0] - 1), DIM == 3 ? min(max(g[1], 0), S.n[1] - 1) : 0,
                            min(max(g[2], 0), S.n[2] - 1));
     }
-    sp.cur[0][p] = X;
-    if (DIM == 3) sp.cur[1][p] = Y;
-    sp.cur[2][p] = Z;
-    sp.cur[3][p] = f64_of(n0);
-    sp.cur[4][p] = f64_of(n1);
-    sp.cur[5][p] = f64_of(n2);
+    sp.dst[0][p] = X;
+    if (DIM == 3) sp.dst[1][p] = Y;
+    sp.dst[2][p] = Z;
+    sp.dst[3][p] = f64_of(n0);
+    sp.dst[4][p] = f64_of(n1);
+    sp.dst[5][p] = f64_of(n2);
     sp.key[p] = key;
     warp_hist_add(sp.count, key);
 }
@@ -2106,7 +2119,16 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     }
                     const JView V = j_view(S, cur);
                     double* sQw = gring;
-                    auto push = [&](int64_t p, const PIn& in) {
+                    const int64_t* const order = PREC == 2 ? hs.order : nullptr;  // (FP32 alone steps indirectly)
+                    auto place = [&](int64_t p) {
+                        if (!order) return p;
+                        // (a step that gave up on a tile load leaves places unset)
+                        const int64_t o = order[p];
+                        return (uint64_t)o < (uint64_t)hs.cap ? o : p;
+                    };
+                    auto push = [&](int64_t p, int64_t src, const PIn& in) {
+                        // an indirect push carries the weight and the id along
+                        const int64_t id = order ? hs.id_src[src] : 0;
                         if constexpr (PREC != 2)
                             push_one_q<R, DIM, ORDER>(s_hot, s_hot.sp[spi], S, cur, sEBd, fx, s_emax, V, sQw,
                                                       s_qtail + warp, s_qhead + warp, P, K.dtd, kq, qsd, p, in,
@@ -2117,6 +2139,10 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         else
                             push_one<R, DIM, ORDER>(s_hot, s_hot.sp[spi], cur, sEB, V, sQw, s_qtail + warp, P,
                                                     K.jf, K.dtd, kq, qs, p, in, sd->err);
+                        if (order) {
+                            hs.dst[6][p] = in.w;
+                            hs.id_dst[p] = id;
+                        }
                     };
                     auto drain_full = [&]() { drain(S, V, K.jf, false); };
                     if constexpr (PPT == 1) {
@@ -2124,19 +2150,22 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         // lane stages its next particle into shared memory with cp.async
                         // one iteration ahead (two buffers per warp, the lane's own column)
                         double* const pbw = smem + P.pb_off + warp * (2 * PIN_SLOTS) + lane;
-                        const int64_t pf = first + lane;
-                        if (P.staged && pf < s1) stage_in<DIM>(s_hot.sp[spi], pf, pbw);
+                        // (indirect: its place is read one iteration before that)
+                        const int64_t bd = blockDim.x, pf = first + lane;
+                        int64_t src = pf < s1 ? place(pf) : 0, nxt = pf + bd < s1 ? place(pf + bd) : 0;
+                        if (P.staged && pf < s1) stage_in<DIM>(hs, src, pbw);
                         cp_async_commit();
                         unsigned buf = 0u;
-                        for (int64_t p0 = first; p0 < s1; p0 += (int64_t)blockDim.x) {
-                            const int64_t pn = p0 + blockDim.x + lane;
-                            if (P.staged && pn < s1) stage_in<DIM>(s_hot.sp[spi], pn, pbw + (buf ^ 1u) * PIN_SLOTS);
-                            cp_async_commit();
-                            cp_async_wait<1>();
+                        for (int64_t p0 = first; p0 < s1; p0 += bd) {
                             const int64_t p = p0 + lane;
+                            if (P.staged && p + bd < s1) stage_in<DIM>(hs, nxt, pbw + (buf ^ 1u) * PIN_SLOTS);
+                            cp_async_commit();
+                            const int64_t after = p + 2 * bd < s1 ? place(p + 2 * bd) : 0;
+                            cp_async_wait<1>();
                             if (p < s1)
-                                push(p, P.staged ? read_staged<DIM>(pbw + buf * PIN_SLOTS)
-                                                 : load_one<DIM>(s_hot.sp[spi], p));
+                                push(p, src, P.staged ? read_staged<DIM>(pbw + buf * PIN_SLOTS) : load_one<DIM>(hs, src));
+                            src = nxt;
+                            nxt = after;
                             buf ^= 1u;
                             drain_full();
                         }
@@ -2144,15 +2173,19 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     } else {
                         for (int64_t p0 = first; p0 < s1; p0 += (int64_t)blockDim.x * PPT) {
                             PIn in[PPT];
+                            int64_t src[PPT];
 #pragma unroll
                             for (int q = 0; q < PPT; ++q) {
                                 const int64_t p = p0 + q * 32 + lane;
-                                if (p < s1) in[q] = load_one<DIM>(s_hot.sp[spi], p);
+                                if (p < s1) {
+                                    src[q] = place(p);
+                                    in[q] = load_one<DIM>(hs, src[q]);
+                                }
                             }
 #pragma unroll
                             for (int q = 0; q < PPT; ++q) {
                                 const int64_t p = p0 + q * 32 + lane;
-                                if (p < s1) push(p, in[q]);
+                                if (p < s1) push(p, src[q], in[q]);
                                 drain_full();
                             }
                         }

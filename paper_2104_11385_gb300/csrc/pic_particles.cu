@@ -144,13 +144,19 @@ __global__ void __launch_bounds__(kScanBlock) pic_scan_final_kernel(SimDev* __re
     }
 }
 
-template <int DIM>
+// INDEX: writes only where each particle is, by sorted place (into the free id
+// buffer): the next push reads through it and writes its particles in sorted
+// order, so the 128 bytes per particle that the full scatter moves are saved in
+// all but the last step of a pic_step call.
+template <int DIM, bool INDEX>
 __global__ void pic_scatter_kernel(SimDev* __restrict__ sims, const int* __restrict__ slots, int sp_idx) {
     const SimDev& S = sims[slots ? slots[blockIdx.y] : 0];
     if (sp_idx < 0) sp_idx = blockIdx.z;
     if (sp_idx >= S.nsp) return;
     const SpeciesDev& sp = S.sp[sp_idx];
     const int64_t np = *sp.np_prev;
+    // an indirect push left the particles in the alternate buffers
+    const bool ind = sp.indirect != 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x; p0 < np; p0 += stride) {
         const int64_t p = p0 + threadIdx.x;
@@ -170,12 +176,18 @@ __global__ void pic_scatter_kernel(SimDev* __restrict__ sims, const int* __restr
         base = __shfl_sync(peers, base, leader);
         int rank = __popc(peers & ((1u << lane) - 1u));
         const int64_t dst = sp.off[k] + base + rank;
+        if constexpr (INDEX) {
+            (ind ? sp.id : sp.id_alt)[dst] = p;
+        } else {
 #pragma unroll
-        for (int a = 0; a < 7; ++a) {
-            if (DIM == 2 && a == 1) continue;
-            sp.alt[a][dst] = sp.cur[a][p];
+            for (int a = 0; a < 7; ++a) {
+                if (DIM == 2 && a == 1) continue;
+                if (ind) sp.cur[a][dst] = sp.alt[a][p];
+                else sp.alt[a][dst] = sp.cur[a][p];
+            }
+            if (ind) sp.id[dst] = sp.id_alt[p];
+            else sp.id_alt[dst] = sp.id[p];
         }
-        sp.id_alt[dst] = sp.id[p];
     }
 }
 
@@ -194,17 +206,23 @@ __global__ void pic_swap_kernel(SimDev* __restrict__ sims, int sp_idx) {
     if (threadIdx.x == 0) swap_buffers(sims[0].sp[sp_idx]);
 }
 
-// end of a step: list heads and step counter, and (swap) the buffers of every
-// species that the step's scatter filled
+// end of a step: list heads, step counter, and each species' buffers after the
+// step's sort.  Full: the sorted particles become current.  Index: the pushed
+// ones do (an indirect push wrote them to the alternate buffers), and the order
+// is then in id_alt.
 __global__ void pic_finish_kernel(SimDev* __restrict__ sims, const int* __restrict__ slots,
-                                  const SchedDev* __restrict__ sd, int swap) {
+                                  const SchedDev* __restrict__ sd, int sort) {
     SimDev& S = sims[slots ? slots[blockIdx.y] : 0];
     if (blockIdx.y == 0) {
         const int nlists = sd->meta[0];
         for (int i = threadIdx.x; i < nlists; i += blockDim.x) sd->head[i] = 0;
     }
     if (threadIdx.x == 0) *S.step += 1;
-    if (swap && (int)threadIdx.x < S.nsp) swap_buffers(S.sp[threadIdx.x]);
+    if (sort != PIC_SORT_NONE && (int)threadIdx.x < S.nsp) {
+        SpeciesDev& sp = S.sp[threadIdx.x];
+        if ((sp.indirect != 0) == (sort == PIC_SORT_INDEX)) swap_buffers(sp);
+        sp.indirect = sort == PIC_SORT_INDEX ? 1 : 0;
+    }
 }
 
 template <int DIM>
@@ -337,8 +355,8 @@ cudaError_t pic_launch_sort(const SimDev* dsim, const SimDev& hsim, int sp, cuda
         pic_scan_kernel<<<1, 1024, 0, st>>>(d, nullptr, sp);
     }
     int64_t cap = hsim.sp[sp].cap;
-    if (hsim.dim == 3) pic_scatter_kernel<3><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
-    else pic_scatter_kernel<2><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
+    if (hsim.dim == 3) pic_scatter_kernel<3, false><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
+    else pic_scatter_kernel<2, false><<<grid_for(cap, 256), 256, 0, st>>>(d, nullptr, sp);
     pic_swap_kernel<<<1, 32, 0, st>>>(d, sp);
     return cudaGetLastError();
 }
@@ -347,7 +365,7 @@ cudaError_t pic_launch_sort(const SimDev* dsim, const SimDev& hsim, int sp, cuda
 // species for large tile counts); the swap of their buffers is left to
 // pic_finish_kernel.  Against three launches per species this takes one launch
 // (one species) to four (two) off a step, about 2 us each where launches count.
-cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, cudaStream_t st) {
+cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, bool index, cudaStream_t st) {
     if (hsim.nsp == 0) return cudaSuccess;
     SimDev* d = const_cast<SimDev*>(dsim);
     const int64_t N = (int64_t)hsim.ntiles + 1;
@@ -364,8 +382,9 @@ cudaError_t pic_launch_sort_all(const SimDev* dsim, const SimDev& hsim, cudaStre
     int64_t cap = 1;
     for (int sp = 0; sp < hsim.nsp; ++sp) cap = std::max(cap, hsim.sp[sp].cap);
     const dim3 g(grid_for(cap, 256), 1, hsim.nsp);
-    if (hsim.dim == 3) pic_scatter_kernel<3><<<g, 256, 0, st>>>(d, nullptr, -1);
-    else pic_scatter_kernel<2><<<g, 256, 0, st>>>(d, nullptr, -1);
+    if (index) pic_scatter_kernel<3, true><<<g, 256, 0, st>>>(d, nullptr, -1);  // either dimensionality
+    else if (hsim.dim == 3) pic_scatter_kernel<3, false><<<g, 256, 0, st>>>(d, nullptr, -1);
+    else pic_scatter_kernel<2, false><<<g, 256, 0, st>>>(d, nullptr, -1);
     return cudaGetLastError();
 }
 
@@ -374,15 +393,15 @@ cudaError_t pic_launch_sort_multi(SimDev* sims, const int* slots, int nslots, in
     if (nslots <= 0) return cudaSuccess;
     pic_scan_kernel<<<dim3(PIC_MAXSP, nslots), 1024, 0, st>>>(sims, slots, -1);
     const dim3 g(grid_for(max_cap, 256) / 4 + 1, nslots, PIC_MAXSP);
-    if (dim == 3) pic_scatter_kernel<3><<<g, 256, 0, st>>>(sims, slots, -1);
-    else pic_scatter_kernel<2><<<g, 256, 0, st>>>(sims, slots, -1);
+    if (dim == 3) pic_scatter_kernel<3, false><<<g, 256, 0, st>>>(sims, slots, -1);
+    else pic_scatter_kernel<2, false><<<g, 256, 0, st>>>(sims, slots, -1);
     return cudaGetLastError();
 }
 
 cudaError_t pic_launch_finish_multi(SimDev* sims, const int* slots, int nslots, const SchedDev* sched,
                                     cudaStream_t st) {
     if (nslots <= 0) return cudaSuccess;
-    pic_finish_kernel<<<dim3(1, nslots), 256, 0, st>>>(sims, slots, sched, 1);
+    pic_finish_kernel<<<dim3(1, nslots), 256, 0, st>>>(sims, slots, sched, PIC_SORT_FULL);
     return cudaGetLastError();
 }
 
@@ -406,8 +425,8 @@ cudaError_t pic_launch_keys_range(const SimDev* dsim, const SimDev& hsim, int sp
     return cudaGetLastError();
 }
 
-cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, bool swap, cudaStream_t st) {
-    pic_finish_kernel<<<1, 256, 0, st>>>(dsim, nullptr, sched, swap ? 1 : 0);
+cudaError_t pic_launch_finish(SimDev* dsim, const SchedDev* sched, int sort, cudaStream_t st) {
+    pic_finish_kernel<<<1, 256, 0, st>>>(dsim, nullptr, sched, sort);
     return cudaGetLastError();
 }
 

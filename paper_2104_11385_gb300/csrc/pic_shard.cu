@@ -487,7 +487,7 @@ pic_status pic_shard_finish(pic_sim* s, int advance) {
     STRY(pic_sim_ensure_ready(s));
     for (int i = 0; i < s->h.nsp; ++i) SCU(s, pic_launch_sort(s->d, s->h, i, s->stream));
     if (advance) {
-        SCU(s, pic_launch_finish(s->d, s->ds, false, s->stream));
+        SCU(s, pic_launch_finish(s->d, s->ds, PIC_SORT_NONE, s->stream));
         s->step_count++;
     }
     STRY(pic_sim_sync(s));

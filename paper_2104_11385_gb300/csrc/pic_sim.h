@@ -57,7 +57,8 @@ struct pic_sim {
     int64_t step_count = 0;
     std::vector<int32_t> box_ijk;
     // graph
-    cudaGraphExec_t graph = nullptr;
+    cudaGraphExec_t graph = nullptr;        // one step
+    cudaGraphExec_t graph_index = nullptr;  // one step that leaves the particles to the next step's push to sort
     bool graph_dirty = true;
     int kernels_per_step = 0;
     // profiling

@@ -132,3 +132,29 @@ def test_bin_positions_at_cell_faces(d):
     assert np.array_equal(off_g, off_r)
     for b in range(len(off_r) - 1):
         assert np.array_equal(np.sort(perm_g[off_r[b]:off_r[b + 1]]), np.sort(perm_r[off_r[b]:off_r[b + 1]]))
+
+
+@pytest.mark.parametrize("dim,order,precision,ppt", [(3, 1, 1, 1), (3, 2, 1, 2), (2, 3, 1, 1), (2, 1, 1, 2), (3, 1, 3, 1),
+                                                     (2, 2, 3, 2)])
+def test_steps_in_one_call_and_one_by_one(dim, order, precision, ppt):
+    """the steps of one call sort through an order, single calls move the particles:
+    the same particles, ids and weights, with some absorbed on the way"""
+    n, b = ((16, 16, 32), (8, 8, 8)) if dim == 3 else ((32, 1, 64), (16, 1, 16))
+    wl = workloads.random_plasma(80, dim, n, b, (0.3, 0.3 if dim == 3 else 1.0, 0.3), order, nspecies=2, npart=5000,
+                                 umax=2.0, absorb=4)
+    wl["species"][1]["w"] *= np.linspace(0.5, 2.0, 5000)
+    fields = workloads.random_fields(3, n, amp=0.2)
+    runs = [make_gpu(wl, fields) for _ in range(3)]
+    for s in runs:
+        s.set_launch(precision=precision, ppt=ppt)
+    runs[0].step(7)
+    for _ in range(7):
+        runs[1].step(1)
+    runs[2].set_lb_params(mode=pic.LB_DYNAMIC, interval=3, theta=0.0, sched=pic.SCHED_QUEUE)
+    for k in (2, 4, 1):
+        runs[2].step(k)
+    tol = 1e-10 if precision == 1 else 3e-5
+    ref = make_oracle(wl, fields)
+    ref.step(7)
+    for s in runs:
+        compare(s, ref, wl, tol=tol)
