@@ -16,9 +16,9 @@
 // takes one warp instruction per SM every 16 clocks, and a particle's gather,
 // push and deposit are 165 FP64 instructions, 2.73 ms at 86 % of that pipe.
 // The gather (60 of them) and the deposit (36) run in 64-bit fixed point on the
-// integer pipes instead (pic_fix.cuh), the Boris push keeps 51: 1.48 ms, about
-// 2600 issued instructions per 32 particles, issue slots 48 % and FP64 pipe
-// 55 % busy (16 warps per SM by registers: latency-bound between the two).  Each thread brackets its particle
+// integer pipes instead (pic_fix.cuh), the Boris push keeps 51: 1.35 ms, about
+// 2700 issued instructions per 32 particles, issue slots 44 % and FP64 pipe
+// 58 % busy (16 warps per SM by registers: latency-bound between the two).  Each thread brackets its particle
 // loop with clock64(); the deltas are warp-reduced, summed in shared memory and
 // added once per unit to the box's cost -- the device-clock cost of
 // arXiv 2104.11385 Sec. 2.2 (Fig. 2a); thread 0 adds the %globaltimer span
@@ -640,9 +640,8 @@ __device__ __forceinline__ double f64_of(float f) {
 // add; a shared FP32 atomic add is a compare-and-swap loop as well, measured
 // at about 2.3 tries per add on the foil, and moving the FP32 variant's
 // current from a shared FP32 tile to these reductions took its particle
-// kernel from 895 to 696 us on the 128^3 foil.)  A float-float value is
-// renormalised and merged to one double first; an FP32 value is widened on its
-// bit pattern (subnormal floats, below 2^-126, become zero).
+// kernel from 895 to 696 us on the 128^3 foil.)  An FP32 value is widened on its bit
+// pattern (subnormal floats, below 2^-126, become zero).
 __device__ __forceinline__ void red_f64(double* p, double v) {
     asm volatile("red.global.add.f64 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "d"(v) : "memory");
 }
@@ -1859,8 +1858,8 @@ struct SimConsts {
 // positions and index math stay FP64 in both, and the current goes to the
 // global FP64 J by L2 reductions).
 // PPT = particles per thread per loop iteration: their HBM loads are issued
-// together before the first of them is pushed (FP32 with PPT 1 stages each
-// lane's next particle through shared memory instead).
+// together before the first of them is pushed (with PPT 1 each lane's
+// next particle is staged through shared memory instead).
 template <int DIM, int ORDER, int MINB, int PREC, int PPT>
 __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev* __restrict__ sd,
                                                               SimDev* __restrict__ sims) {
