@@ -523,7 +523,7 @@ pic_status capture_one(pic_sim* s, bool index, cudaGraphExec_t* out) {
 pic_status capture_graph(pic_sim* s) {
     drop_graphs(s);
     TRY(capture_one(s, false, &s->graph));
-    TRY(capture_one(s, true, &s->graph_index));
+    if (s->prec == 2) TRY(capture_one(s, true, &s->graph_index));  // (pic_step: FP32 alone uses it)
     s->graph_dirty = false;
     s->kernels_per_step = count_kernels(s);
     return PIC_OK;
