@@ -51,9 +51,9 @@ __device__ __forceinline__ int bin_div(int i, int b, float rb) {
 
 __device__ __forceinline__ int bin_box_of(const BinGeom& g, const double* x, const double* y,
                                           const double* z, int64_t p) {
-    const int cx = bin_div(bin_cell(x[p], g.d[0], g.inv[0], g.n[0]), g.bsz[0], 1.0f / (float)g.bsz[0]);
-    const int cy = g.dim == 3 ? bin_div(bin_cell(y[p], g.d[1], g.inv[1], g.n[1]), g.bsz[1], 1.0f / (float)g.bsz[1]) : 0;
-    const int cz = bin_div(bin_cell(z[p], g.d[2], g.inv[2], g.n[2]), g.bsz[2], 1.0f / (float)g.bsz[2]);
+    const int cx = bin_div(bin_cell(x[p], g.d[0], g.inv[0], g.n[0]), g.bsz[0], g.rbsz[0]);
+    const int cy = g.dim == 3 ? bin_div(bin_cell(y[p], g.d[1], g.inv[1], g.n[1]), g.bsz[1], g.rbsz[1]) : 0;
+    const int cz = bin_div(bin_cell(z[p], g.d[2], g.inv[2], g.n[2]), g.bsz[2], g.rbsz[2]);
     return (cz * g.nb[1] + cy) * g.nb[0] + cx;
 }
 
@@ -151,6 +151,7 @@ pic_status pic_bin_validate(const pic_grid_desc* grid, const double* x, const do
         g->nb[a] = g->n[a] / g->bsz[a];
         g->d[a] = act ? grid->dx[a] : 1.0;
         g->inv[a] = std::isnormal(1.0 / g->d[a]) ? 1.0 / g->d[a] : NAN;  // NaN: always divide
+        g->rbsz[a] = 1.0f / (float)g->bsz[a];
         nboxes *= g->nb[a];
     }
     if (nboxes > (int64_t)1 << 30) {

@@ -12,6 +12,7 @@ struct BinGeom {
     int dim;
     int n[3], bsz[3], nb[3];
     double d[3], inv[3];  // cell sizes and their reciprocals
+    float rbsz[3];        // reciprocals of the box extents
     int nboxes;
 };
 
