@@ -70,6 +70,24 @@ __global__ void bin_count_kernel(BinGeom g, const double* __restrict__ x, const 
     }
 }
 
+// The same through a histogram in shared memory per CTA, added to the global one
+// at the end: for many particles per box (bin_shared).
+constexpr int kBinHistMax = 8192;  // boxes: 32 KB
+__global__ void __launch_bounds__(1024) bin_count_shared_kernel(BinGeom g, const double* __restrict__ x,
+                                                                const double* __restrict__ y,
+                                                                const double* __restrict__ z, int64_t np,
+                                                                unsigned long long* __restrict__ off) {
+    __shared__ int hist[kBinHistMax];
+    for (int b = threadIdx.x; b < g.nboxes; b += blockDim.x) hist[b] = 0;
+    __syncthreads();
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += stride)
+        atomicAdd(hist + bin_box_of(g, x, y, z, p), 1);
+    __syncthreads();
+    for (int b = threadIdx.x; b < g.nboxes; b += blockDim.x)
+        if (hist[b] != 0) atomicAdd(off + b + 1, (unsigned long long)hist[b]);
+}
+
 // in-place exclusive scan of off[1..nboxes] (off[0] = 0) by one CTA
 __global__ void __launch_bounds__(1024) bin_scan_kernel(int64_t* __restrict__ off, int nboxes) {
     __shared__ int64_t part[1024];
@@ -111,6 +129,10 @@ __global__ void bin_scatter_kernel(BinGeom g, const double* __restrict__ x, cons
         perm[off[b] + base + __popc(peers & ((1u << lane) - 1u))] = p;
     }
 }
+
+// the shared histograms pay when adding them up takes at most a quarter of the
+// global atomics they save
+bool bin_shared(int nboxes, int64_t np, int ctas) { return nboxes <= kBinHistMax && np >= 4ll * ctas * nboxes; }
 
 int bin_grid(int64_t np) {
     int64_t b = (np + 255) / 256;
@@ -168,7 +190,10 @@ cudaError_t pic_bin_launch(const BinGeom& g, const double* x, const double* y, c
     cudaError_t e = cudaMemsetAsync(box_off, 0, (size_t)(g.nboxes + 1) * sizeof(int64_t), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, (size_t)g.nboxes * sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
-    if (np > 0)
+    const int wide = 2 * pic_sm_count();  // CTAs of 1024 threads, two per SM
+    if (np > 0 && bin_shared(g.nboxes, np, wide))
+        bin_count_shared_kernel<<<wide, 1024, 0, st>>>(g, x, y, z, np, (unsigned long long*)box_off);
+    else if (np > 0)
         bin_count_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, (unsigned long long*)box_off);
     bin_scan_kernel<<<1, 1024, 0, st>>>(box_off, g.nboxes);
     if (np > 0) bin_scatter_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
