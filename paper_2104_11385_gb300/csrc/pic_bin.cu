@@ -130,8 +130,48 @@ __global__ void bin_scatter_kernel(BinGeom g, const double* __restrict__ x, cons
     }
 }
 
+// The scatter for the same inputs: a CTA ranks 16 positions per thread in shared
+// memory and takes one global cursor step per box it met instead of one per
+// position (a returning atomic each, contended where boxes are few).  Per call:
+// 1 M positions in 512 boxes 156 -> 57 us, 16.8 M in 4096 boxes 704 -> 589 us
+// shuffled and 857 -> 534 ordered along z.
+constexpr int kBinPer = 16;
+__global__ void __launch_bounds__(1024) bin_scatter_shared_kernel(BinGeom g, const double* __restrict__ x,
+                                                                  const double* __restrict__ y,
+                                                                  const double* __restrict__ z, int64_t np,
+                                                                  const int64_t* __restrict__ off,
+                                                                  int32_t* __restrict__ cursor,
+                                                                  int64_t* __restrict__ perm) {
+    __shared__ int hist[kBinHistMax];
+    const int64_t chunk = (int64_t)kBinPer * blockDim.x;
+    for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < np; c0 += (int64_t)gridDim.x * chunk) {
+        for (int b = threadIdx.x; b < g.nboxes; b += blockDim.x) hist[b] = 0;
+        __syncthreads();
+        int box[kBinPer], rank[kBinPer];
+#pragma unroll
+        for (int k = 0; k < kBinPer; ++k) {
+            const int64_t p = c0 + (int64_t)k * blockDim.x + threadIdx.x;
+            box[k] = -1;
+            if (p < np) {
+                box[k] = bin_box_of(g, x, y, z, p);
+                rank[k] = atomicAdd(hist + box[k], 1);
+            }
+        }
+        __syncthreads();
+        for (int b = threadIdx.x; b < g.nboxes; b += blockDim.x)
+            if (hist[b] != 0) hist[b] = atomicAdd(cursor + b, hist[b]);
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < kBinPer; ++k)
+            if (box[k] >= 0)
+                perm[off[box[k]] + hist[box[k]] + rank[k]] = c0 + (int64_t)k * blockDim.x + threadIdx.x;
+        __syncthreads();
+    }
+}
+
 // the shared histograms pay when adding them up takes at most a quarter of the
-// global atomics they save
+// global atomics they save (counts of 16.8 M positions in 4096 boxes: 803 -> 704
+// us per call; 100 thousand positions there stay with the global ones, 31 us)
 bool bin_shared(int nboxes, int64_t np, int ctas) { return nboxes <= kBinHistMax && np >= 4ll * ctas * nboxes; }
 
 int bin_grid(int64_t np) {
@@ -196,7 +236,10 @@ cudaError_t pic_bin_launch(const BinGeom& g, const double* x, const double* y, c
     else if (np > 0)
         bin_count_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, (unsigned long long*)box_off);
     bin_scan_kernel<<<1, 1024, 0, st>>>(box_off, g.nboxes);
-    if (np > 0) bin_scatter_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
+    if (np > 0 && bin_shared(g.nboxes, np, wide))
+        bin_scatter_shared_kernel<<<wide, 1024, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
+    else if (np > 0)
+        bin_scatter_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
     return cudaGetLastError();
 }
 

@@ -158,3 +158,23 @@ def test_steps_in_one_call_and_one_by_one(dim, order, precision, ppt):
     ref.step(7)
     for s in runs:
         compare(s, ref, wl, tol=tol)
+
+
+@pytest.mark.parametrize("npart", [9727, 9728, 16384, 16385, 5000003])  # 8 boxes: shared-memory counts from 9728 on (152 SMs)
+@pytest.mark.parametrize("one_box", [False, True])
+def test_bin_shared_counts(npart, one_box):
+    import torch
+    from paper_2104_11385_gb300 import sim as S
+    n, box, d = (16, 16, 16), (8, 8, 8), 0.3
+    r = np.random.default_rng(npart)
+    x, y, z = (r.uniform(0.0, (8 if one_box else 16) * d * 0.999, npart) for _ in range(3))
+    off = torch.empty(9, dtype=torch.int64, device="cuda")
+    perm = torch.empty(npart, dtype=torch.int64, device="cuda")
+    S.bin_particles(3, n, box, (d, d, d), *(torch.as_tensor(a, device="cuda") for a in (x, y, z)), off, perm)
+    torch.cuda.synchronize()
+    cell = [np.floor(a / d).astype(np.int64) // 8 for a in (x, y, z)]
+    want = (cell[2] * 2 + cell[1]) * 2 + cell[0]
+    off_g, perm_g = off.cpu().numpy(), perm.cpu().numpy()
+    assert np.array_equal(off_g, np.concatenate([[0], np.cumsum(np.bincount(want, minlength=8))]))
+    assert np.array_equal(want[perm_g], np.repeat(np.arange(8), np.diff(off_g)))
+    assert np.array_equal(np.sort(perm_g), np.arange(npart))
