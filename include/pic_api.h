@@ -345,16 +345,20 @@ pic_status pic_bin_particles(const pic_grid_desc* grid, const double* x, const d
  *   ppt           particles per thread per loop iteration (1 or 2): the HBM
  *                 loads of that many particles are issued before the first
  *                 of them is pushed.
- *   precision     arithmetic of the particle push: 1 FP64 (default);
- *                 2 float-float or better (a significand of at least 48 bits
- *                 for gather, Boris and deposit weights): runs the arithmetic
- *                 of 1, which is the faster of the two; 3 FP32
- *                 for gather, Boris and deposit weights with FP64 storage,
- *                 positions and current accumulation (the FP32 variant:
- *                 about 2^-24 per operation, so it meets an FP32-derived
- *                 tolerance, not the FP64 one); 0 keeps the current
- *                 setting.  The autotuner
- *                 never changes it. */
+ *   precision     arithmetic of the particle push: 1 FP64 (default): the Boris
+ *                 push in FP64, gather and deposit in 64-bit fixed point.  A
+ *                 gathered component is within 2^-51 of the strongest field
+ *                 value it is interpolated from, or, where all of those lie
+ *                 below 2^-4 (linear shapes) or 2^-2 (others) of the
+ *                 component's largest magnitude in the staged tile, within
+ *                 2^-46; below 2^-10 (2^-8) of it FP64 takes over;
+ *                 2 float-float or better: runs the arithmetic of 1, which is
+ *                 the faster of the two;
+ *                 3 FP32 for gather, Boris and deposit weights with FP64
+ *                 storage, positions and current accumulation (the FP32
+ *                 variant: about 2^-24 per operation, so it meets an
+ *                 FP32-derived tolerance, not the FP64 one);
+ *                 0 keeps the current setting.  The autotuner never changes it. */
 typedef struct {
     int threads, ctas_per_sm, split, precision, tile, ppt;
 } pic_launch_cfg;

@@ -12,7 +12,10 @@
 //   Q62     a weight, an offset or a move in cells, in units of 2^-62
 //   tile    a field value in units of 2^(e - FB), 2^e > every magnitude of that
 //           component in the tile; FB = 62 for linear shapes, 60 for the
-//           others (headroom of the row sums)
+//           others (headroom of the row sums).  A value down to 2^-9 (2^-7) of
+//           the largest keeps a double's 53 bits, a smaller one fewer: the tile's
+//           cells where a component is weak are marked when it is staged
+//           (weak_limit), and their particles gather it in FP64
 //   Amp     a floating-point factor: 64-bit mantissa, exponent, sign
 // Only the last step of each chain returns to IEEE doubles, by bit operations
 // and with one rounding: the six field values, and every current contribution.
@@ -241,12 +244,28 @@ __device__ __forceinline__ SupQ<ORDER> half_support(const CellQ& c, int o, bool 
 // ---- tile values ----------------------------------------------------------
 template <int ORDER>
 struct TileBits {
-        static constexpr int FB = ORDER == 1 ? 62 : 60;
+    static constexpr int FB = ORDER == 1 ? 62 : 60;
 };
 // biased exponent of the largest magnitude of a component: 0 (all zeros or
 // subnormal, held as zero) or within these bounds; a tile outside them (Inf and
 // NaN among others) is gathered in FP64
 __device__ __forceinline__ bool tile_exp_ok(int e) { return e == 0 || (e >= 128 && e <= 1900); }
+
+// The weakest field that is gathered in fixed point, as the high word of a double:
+// 2^-10 (linear) or 2^-8 of the component's largest magnitude in the tile.  Error
+// of the gather against exact arithmetic, relative to the strongest node it
+// interpolates from, random nodes (rms, largest):
+//                           linear 3D            cubic 3D
+//   nodes near the largest  1.5e-17, 1.0e-16     8.4e-18, 5.7e-17
+//   nodes at the limit      1.7e-15, 1.4e-14     1.4e-15, 7.5e-15
+//   FP64                    3.7e-17, 3.9e-16     3.7e-17, 3.5e-16
+// so a weak place keeps 46 bits or more, and FP64's where it is weaker still.  A
+// laser on a foil has whole layers between 2^-7 and 2^-10 behind the skin: a limit
+// of 2^-7 costs the 256^3 foil 30 % of its particle kernel there, 2^-10 1 %.
+template <int ORDER>
+__device__ __forceinline__ unsigned weak_limit(int emax) {
+    return (unsigned)(emax - (ORDER == 1 ? 10 : 8)) << 20;
+}
 
 // a double in units of 2^(emax - 1022 - FB), rounded to nearest; emax: biased
 // exponent of the component's largest magnitude

@@ -264,10 +264,10 @@ struct EBHalo {
     static constexpr int lo = ORDER == 3 ? 2 : 1;
 };
 
-// interpolation of one component from a shared tile of R values (FP32, and FP64
-// for tiles that the fixed-point gather does not take) with extents (SX, SY)
-template <class R, int ORDER, int DIM>
-__device__ __forceinline__ R interp(const R* __restrict__ F, int SX, int SY, const Support<ORDER, R>& sx,
+// interpolation of one component from R values with extents (SX, SY): a shared
+// tile (FP32), or in FP64 the global arrays (I = int64_t)
+template <class R, int ORDER, int DIM, class I>
+__device__ __forceinline__ R interp(const R* __restrict__ F, I SX, I SY, const Support<ORDER, R>& sx,
                                     const Support<ORDER, R>& sy, const Support<ORDER, R>& sz) {
     // tile column 0 is local cell -EBHalo<ORDER>::lo
     constexpr int H = EBHalo<ORDER>::lo;
@@ -385,25 +385,109 @@ __device__ __forceinline__ Six gather6_q(const long long* __restrict__ F, int st
     return r;
 }
 
-// the same in FP64 from the doubles as staged: tiles holding Inf or NaN, or
-// magnitudes outside the fixed-point gather's exponent range
+// Component c of the same in FP64 from the global arrays (which the kernel only
+// reads), out of line: for particles in cells where it is marked as weak.
 template <int ORDER, int DIM>
-static __device__ __noinline__ Six gather6_fp64(const double* __restrict__ sEB, int stride, int SX, int SY, double X,
-                                                double Y, double Z, int ox, int oy, int oz, bool ec) {
-    Support<ORDER, double> nd[3], hf[3];
-    int c;
-    supports_at<ORDER, double>(X, ox, ec, nd[0], hf[0], c);
-    supports_at<ORDER, double>(Z, oz, ec, nd[2], hf[2], c);
-    if (DIM == 3) {
-        supports_at<ORDER, double>(Y, oy, ec, nd[1], hf[1], c);
+static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, double X, double Y, double Z, int ox, int oy,
+                                                   int oz) {
+    constexpr int H = EBHalo<ORDER>::lo;
+    const bool ec = S.ec != 0, isb = c >= 3;
+    const int a = isb ? c - 3 : c;
+    auto one = [&](double x, int o, bool half) {
+        Support<ORDER, double> nd, hf;
+        int cell;
+        supports_at<ORDER, double>(x, o, ec, nd, hf, cell);
+        return half ? hf : nd;
+    };
+    const Support<ORDER, double> sx = one(X, ox, (a == 0) != isb), sz = one(Z, oz, (a == 2) != isb);
+    Support<ORDER, double> sy = sx;
+    if (DIM == 3) sy = one(Y, oy, (a == 1) != isb);
+    const double* F = S.F[c] + pidx(S, ox - H, DIM == 3 ? oy - H : 0, oz - H);
+    if constexpr (ORDER == 1) {
+        return interp<double, ORDER, DIM, int64_t>(F, S.pn[0], S.pn[1], sx, sy, sz);
     } else {
-        nd[1].s = -1;
-        nd[1].w[0] = 1.0;
-        hf[1] = nd[1];
+        // rolled, few registers: what a call clobbers is spilled around it on the
+        // caller's fast path too (unrolled, the cubic kernel spills 500 bytes)
+        double v = 0.0;
+#pragma unroll 1
+        for (int k = 0; k <= ORDER; ++k) {
+            double pl = 0.0;
+#pragma unroll 1
+            for (int j = 0; j <= (DIM == 3 ? ORDER : 0); ++j) {
+                const double* row =
+                    F + ((sz.s + H + k) * (int64_t)S.pn[1] + (DIM == 3 ? sy.s + H + j : 0)) * S.pn[0] + sx.s + H;
+                double l = 0.0;
+#pragma unroll
+                for (int i = 0; i <= ORDER; ++i) l = fma(sx.w[i], row[i], l);
+                pl = DIM == 3 ? fma(sy.w[j], l, pl) : l;
+            }
+            v = fma(sz.w[k], pl, v);
+        }
+        return v;
     }
-    Six r;
-    gather6<double, ORDER, DIM>(sEB, stride, SX, SY, nd, hf, r.v, r.v + 3);
-    return r;
+}
+
+// Marks the cells of a staged tile where a component is gathered in FP64: bits +
+// c * words, one bit per tile element.  Every 2 x 2 x 2 nodes of a component (a
+// single node along the half-node directions of the energy-conserving linear
+// gather) must reach weak_limit or be all zero; if not, the cells whose particles
+// interpolate from them are marked: the one at their lower corner, and along a
+// half-node direction the next one too.  (Quadratic shapes: the cell of nearest
+// node.  All orders have those nodes in their particles' supports.)  Linear shapes look at 4 of
+// the 8 nodes, the others, whose limit is higher, at all.  Elements are taken in a
+// row across row ends (what that marks needlessly lies in the halo), 31 windows
+// per warp and round, the components side by side: the shuffle gives the nodes one
+// further in x.  About 1 us per staged tile and CTA (16^3 plasma 40.0 -> 41.2 us
+// per step, 128^3 foil 1365 -> 1393 with the test of the marks, quadratic
+// log-normal boxes 4505 -> 4633).
+template <int ORDER, int DIM>
+__device__ __forceinline__ bool mark_weak(unsigned* __restrict__ bits, int words, const double* __restrict__ sEB,
+                                          int stride, int vol, int SX, int SY, const int* __restrict__ emax, bool ec) {
+    const int lane = threadIdx.x & 31, SZ = DIM == 3 ? SX * SY : SX;
+    const bool one = ORDER == 1 && ec;
+    unsigned lim[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) lim[c] = emax[c] == 0 ? 0u : weak_limit<ORDER>(emax[c]);
+    const int n = vol - SZ - (DIM == 3 ? SX : 0);  // windows that lie in the tile
+    bool any = false;
+    for (int i0 = (threadIdx.x >> 5) * 31; i0 < n; i0 += (blockDim.x >> 5) * 31) {
+        const int i = min(i0 + lane, n - 1);
+        unsigned weak = 0u;
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const int a = c < 3 ? c : c - 3;
+            const bool isb = c >= 3, hx = (a == 0) != isb, hy = (a == 1) != isb, hz = (a == 2) != isb;
+            const int dy = DIM == 2 || (one && hy) ? 0 : SX, dz = one && hz ? 0 : SZ;
+            const unsigned* h = reinterpret_cast<const unsigned*>(sEB + c * stride) + 1;  // high words
+            auto mag = [&](int k) { return h[2 * k] & 0x7FFFFFFFu; };
+            unsigned m = max(mag(i), mag(i + dy + dz));
+            if (DIM == 3 && (ORDER > 1 || one)) m = max(m, max(mag(i + dy), mag(i + dz)));
+            const unsigned mx = __shfl_down_sync(0xffffffffu, m, 1);
+            if (!(one && hx)) m = max(m, mx);
+            weak |= m != 0u && m < lim[c] ? 1u << c : 0u;
+        }
+        if (lane == 31 || i0 + lane >= n) weak = 0u;
+        if (__any_sync(0xffffffffu, weak != 0u)) {
+            any = true;
+#pragma unroll 1
+            for (int c = 0; c < 6; ++c) {
+                const unsigned w = __ballot_sync(0xffffffffu, (weak >> c) & 1u);
+                if (w == 0u) continue;
+                const int a = c < 3 ? c : c - 3;
+                const bool isb = c >= 3, hx = (a == 0) != isb, hy = DIM == 3 && ((a == 1) != isb), hz = (a == 2) != isb;
+                // lane: along which of the half-node directions the marked cell is the next one
+                if (lane < 8 && (!(lane & 1) || (hx && !one)) && (!(lane & 2) || (hy && !one)) &&
+                    (!(lane & 4) || (hz && !one))) {
+                    const int b = i0 + (lane & 1 ? 1 : 0) + (lane & 2 ? SX : 0) + (lane & 4 ? SZ : 0);
+                    const unsigned up = (b & 31) ? w >> (32 - (b & 31)) : 0u;
+                    unsigned* const to = bits + c * words + (b >> 5);
+                    if ((b >> 5) < words) atomicOr(to, w << (b & 31));
+                    if (up != 0u && (b >> 5) + 1 < words) atomicOr(to + 1, up);
+                }
+            }
+        }
+    }
+    return any;
 }
 
 // Esirkepov node shapes on a common window of W nodes starting at the lower of
@@ -591,6 +675,8 @@ struct SmemPlan {
     int eb_stride;  // doubles per E/B component (multiple of 16 -> 128-byte aligned)
     int eb_vol;
     int pb_off;     // doubles from the base to the particle staging buffers
+    int bit_off;    // doubles from the base to the marks of weak cells
+    int bit_words;  // words of them per component
     bool staged;    // whether there are such buffers
     size_t bytes;
 };
@@ -603,7 +689,7 @@ constexpr int PIC_PBUF_DOUBLES = QMAXWARPS * 2 * PIN_SLOTS;
 // FP64 converts the staged E/B tile in place to fixed point, the FP32 variant for linear
 // shapes to float pairs (F[x], F[x+1] - F[x]), component c at pair c *
 // eb_stride, otherwise to floats, component c at float c * eb_stride.
-// Layout: E/B tile (TMA) | particle buffers.
+// Layout: E/B tile (TMA) | particle buffers | marks of weak cells.
 __host__ __device__ inline SmemPlan smem_plan(const int ebs[3]) {
     SmemPlan p;
     p.eb_vol = ebs[0] * ebs[1] * ebs[2];
@@ -611,8 +697,11 @@ __host__ __device__ inline SmemPlan smem_plan(const int ebs[3]) {
     p.pb_off = 6 * p.eb_stride;
     // tiles too large to leave room for the buffers (2D tiles of 64 cells) load
     // their particles directly
-    p.staged = (p.pb_off + PIC_PBUF_DOUBLES) * sizeof(double) <= 225 * 1024;
-    p.bytes = (size_t)(p.pb_off + (p.staged ? PIC_PBUF_DOUBLES : 0)) * sizeof(double);
+    p.bit_words = (p.eb_vol + 31) / 32;
+    const int bits = 3 * p.bit_words;  // doubles that 6 components' words take
+    p.staged = (p.pb_off + PIC_PBUF_DOUBLES + bits) * sizeof(double) <= 225 * 1024;
+    p.bit_off = p.pb_off + (p.staged ? PIC_PBUF_DOUBLES : 0);
+    p.bytes = (size_t)(p.bit_off + bits) * sizeof(double);
     return p;
 }
 
@@ -1291,11 +1380,12 @@ __device__ __forceinline__ PIn read_staged(const double* slot) {
 }
 
 // Gather, Boris push, and deposit of one particle, FP64.  The gather and the
-// deposit are fixed-point; fx: the staged tile is in fixed point (emax: biased
-// exponents per component), otherwise it holds the doubles as loaded.
+// deposit are fixed-point; emax: biased exponents of the staged tile's components;
+// weak: its cells where a component is gathered in FP64, nullptr if there is none.
 template <class R, int DIM, int ORDER, class SV, class SPV>
 __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const SimDev& SG, const Tile& tl,
-                                           const double* __restrict__ sEB, bool fx, const int* __restrict__ emax,
+                                           const double* __restrict__ sEB, const unsigned* weak,
+                                           const int* __restrict__ emax,
                                            const JView& V, double* __restrict__ sQw, unsigned* s_one, unsigned* s_many,
                                            const SmemPlan& P, const R* dtd, R kq, double qs, int64_t p, const PIn& in,
                                            int32_t* err) {
@@ -1326,12 +1416,20 @@ __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const Sim
             warp_hist_add(sp.count, S.ntiles);
             return;
         }
-        if (fx)
-            f = gather6_q<ORDER, DIM>(reinterpret_cast<const long long*>(sEB), P.eb_stride, S.ebs[0], S.ebs[1], emax,
-                                      na, ha);
-        else
-            f = gather6_fp64<ORDER, DIM>(sEB, P.eb_stride, S.ebs[0], S.ebs[1], x0[0], x0[1], x0[2], tl.o[0], tl.o[1],
-                                         tl.o[2], S.ec != 0);
+        f = gather6_q<ORDER, DIM>(reinterpret_cast<const long long*>(sEB), P.eb_stride, S.ebs[0], S.ebs[1], emax, na, ha);
+        if (weak) {
+            // the particle's cell (quadratic: its nearest node)
+            constexpr int B = EBHalo<ORDER>::lo + (ORDER == 1 ? 0 : 1);
+            const int i = ((nd[2].s + B) * S.ebs[1] + (DIM == 3 ? nd[1].s + B : 0)) * S.ebs[0] + nd[0].s + B;
+            weak += i >> 5;
+#pragma unroll 1
+            for (int c = 0; c < 6; ++c, weak += P.bit_words) {
+                if (((*weak >> (i & 31)) & 1u) == 0u) continue;
+                const double v = gather1_fp64<ORDER, DIM>(SG, c, x0[0], x0[1], x0[2], tl.o[0], tl.o[1], tl.o[2]);
+#pragma unroll
+                for (int k = 0; k < 6; ++k) f.v[k] = c == k ? v : f.v[k];
+            }
+        }
         if (nan) f.v[0] = f.v[1] = f.v[2] = __longlong_as_double(0x7FF8000000000000ll);
     }
     const R u0 = A::from(in.u0), u1 = A::from(in.u1), u2 = A::from(in.u2);
@@ -1874,6 +1972,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
     __shared__ unsigned s_qhead[QMAXWARPS], s_qtail[QMAXWARPS];
     __shared__ unsigned long long s_cost, s_time;
     __shared__ int s_emax[6];  // fixed-point tile: biased exponent of each component's largest magnitude
+    __shared__ int s_some;     // whether a cell is marked as too weak for it (mark_weak)
 
     const int nlists = sd->meta[0];
     const int steal = sd->meta[1];
@@ -1891,7 +1990,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
     cur.sim = -1;
     cur.t = -1;
     int visited = 0, hot = -1;
-    bool fx = false;  // the staged tile is in fixed point
+    const unsigned* weak = nullptr;  // the marks, if the staged tile has such cells
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // ring of cell-crossing particles, in global scratch (L1/L2 resident; a
     // drain runs once per 32 crossings)
@@ -1958,6 +2057,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
         const bool cap_clk = (S.capture & 1) != 0, cap_time = (S.capture & 2) != 0;
         const SmemPlan P = smem_plan(S.ebs);
         double* sEBd = smem;
+        unsigned* const s_bits = reinterpret_cast<unsigned*>(smem + P.bit_off);
         const R* sEB = reinterpret_cast<const R*>(smem);
         unsigned long long my_clk = 0ull;
         const SimConsts<R, DIM> K(S);
@@ -2008,6 +2108,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     tile_origin(S, t, cur.o);
                     if (threadIdx.x == 0) {
                         for (int c = 0; c < 6; ++c) s_emax[c] = 0;
+                        s_some = 0;
                         fence_proxy_async();
                         mbar_expect_tx(&bar, (uint32_t)(6 * P.eb_vol * sizeof(double)));
                         constexpr int H = EBHalo<ORDER>::lo;
@@ -2018,6 +2119,8 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         for (int c = 0; c < 6; ++c)
                             tma_load_3d(sEBd + c * P.eb_stride, &S.tmap[c], x0, y0, z0, &bar);
                     }
+                    if (PREC != 2)
+                        for (int i = threadIdx.x; i < 6 * P.bit_words; i += blockDim.x) s_bits[i] = 0u;
                     for (int i = threadIdx.x; i < 9; i += blockDim.x) {
                         const int a = i / 3, side = i - 3 * a;
                         const int c = a == 0 ? cur.o[0] : (a == 1 ? cur.o[1] : cur.o[2]);
@@ -2048,8 +2151,18 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                             if (lane == 0) atomicMax(&s_emax[c], (int)(mx >> 20));
                         }
                         __syncthreads();
-                        fx = true;
+                        bool fx = true;
                         for (int c = 0; c < 6; ++c) fx = fx && tile_exp_ok(s_emax[c]);
+                        if (fx) {
+                            if (mark_weak<ORDER, DIM>(s_bits, P.bit_words, sEBd, P.eb_stride, P.eb_vol, S.ebs[0], S.ebs[1],
+                                                      s_emax, S.ec != 0))
+                                s_some = 1;
+                        } else {  // every cell: Inf, NaN, or magnitudes outside the exponent range
+                            for (int i = threadIdx.x; i < 6 * P.bit_words; i += blockDim.x) s_bits[i] = ~0u;
+                            s_some = 1;
+                        }
+                        __syncthreads();
+                        weak = s_some ? s_bits : nullptr;
                         if (fx) {
                             for (int c = 0; c < 6; ++c) {
                                 const int em = s_emax[c];
@@ -2129,7 +2242,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         // an indirect push carries the weight and the id along
                         const int64_t id = order ? hs.id_src[src] : 0;
                         if constexpr (PREC != 2)
-                            push_one_q<R, DIM, ORDER>(s_hot, s_hot.sp[spi], S, cur, sEBd, fx, s_emax, V, sQw,
+                            push_one_q<R, DIM, ORDER>(s_hot, s_hot.sp[spi], S, cur, sEBd, weak, s_emax, V, sQw,
                                                       s_qtail + warp, s_qhead + warp, P, K.dtd, kq, qsd, p, in,
                                                       sd->err);
                         else if constexpr (ORDER == 1)
