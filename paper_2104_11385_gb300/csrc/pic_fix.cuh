@@ -101,6 +101,7 @@ struct AccQ {
 };
 __device__ __forceinline__ q62 mulq(const Limb& a, const Limb& b) {
     AccQ s;
+    s.mid = 1ll << 29;  // to nearest
     s.mac(a, b);
     return s.get();
 }
@@ -118,23 +119,21 @@ __device__ __forceinline__ u64 mulhi(u64 a, u64 b) {
     return mad_uu(ah, bh, mid >> 32);
 }
 
-// |v| 2^x as an IEEE double's magnitude: hi is the exponent part of its high
-// word, (x + 1085) << 20 (with a sign bit, if any); v != 0 or the result is
-// meaningless.  ROUND: to nearest, else toward zero.
+// v 2^x as an IEEE double, v < 2^63, rounded to nearest (ROUND) or toward zero: hi is the exponent part of
+// its high word, (x + 1085) << 20 (with a sign bit, if any); v != 0 or the result
+// is meaningless.
 template <bool ROUND>
 __device__ __forceinline__ double pack_double(u64 v, unsigned hi) {
     unsigned h = (unsigned)(v >> 32), lo = (unsigned)v;
     if (h == 0u) {
-        h = lo;
-        lo = 0u;
-        hi -= 32u << 20;
+        h = lo >> 1;
+        lo <<= 31;
+        hi -= 31u << 20;
     }
     const int l = __clz((int)h);
-    const unsigned mh = __funnelshift_l(lo, h, l), ml = lo << (l & 31);  // leading one in bit 63
-    u64 m = ((u64)mh << 32) | ml;
+    // leading one in bit 62: the half unit that rounds cannot carry out
+    const u64 m = ((((u64)__funnelshift_l(lo, h, l - 1) << 32) | (lo << (l - 1))) + (ROUND ? 0x200u : 0u)) >> 10;
     // (53 bits: the leading one adds 1 to the exponent field)
-    if (ROUND) m = (m >> 11) + ((ml >> 10) & 1u);
-    else m >>= 11;
     return __longlong_as_double((long long)(((u64)((unsigned)(m >> 32) + hi - ((unsigned)l << 20)) << 32) | (unsigned)m));
 }
 
@@ -366,6 +365,15 @@ __device__ __forceinline__ Amp amp_scale(const Amp& a, q62 p) {
     const int l = __clz((int)h);
     const u64 n = ((u64)__funnelshift_l(lo, h, l) << 32) | (lo << (l & 31));
     return Amp{v == 0ull ? 0ull : mulhi(a.m, n >> 1), es - ((unsigned)l << 20)};
+}
+// A current contribution, amplitude x weight, rounded to nearest; false if there
+// is none: a weight of zero, or a few units below it by the roundings of its
+// factors.  Beside that rounding mulhi drops up to 2 units of 2^(e + 2): a
+// current's amplitudes have m >= 2^58, so that is at most 2^-55 of the amplitude.
+__device__ __forceinline__ bool contribution(const Amp& a, q62 T, double& v) {
+    const u64 jm = mulhi(a.m, (u64)T);  // value jm 2^(e + 2)
+    v = pack_double<true>(jm, a.es + (1087u << 20));
+    return (int)(T >> 32) >= 0 && jm != 0ull;
 }
 // the exponent fields of a factor q w whose product with any of three
 // prefactors, and every contribution of that, is a normal double (lo > hi: none)

@@ -958,16 +958,15 @@ __device__ __forceinline__ void deposit_lin_incell_d(const SV& S, const JView& V
 // A contribution is amplitude x weight: the weight (the transverse factor, in
 // [0, 1]) is a Q62 number, the amplitude (prefactor, q w and the prefix sum of
 // DS along the current's direction, or v_y in 2D) an Amp; their product is
-// rounded once, to the double that goes to L2.  Against FP64 factors this takes
-// the deposit off the FP64 pipe (36 of about 165 FP64 instructions per particle
-// for linear shapes) and rounds each contribution once instead of four to six
-// times.
-//
-// T >= 0.  The contribution is rounded toward zero (at most 2^-52 of it, where
-// the FP64 factors took four to six roundings of 2^-53 each).
+// rounded once, to the double that goes to L2.  The weight is good to 8 units of
+// 2^-62 (24 for cubic shapes), so a contribution is within 2^-53 of itself and
+// 2^-54 of its amplitude, which is what 1 - m alone costs the FP64 factors and
+// their four to six roundings.  Nodes that only small weights reach have that
+// absolute accuracy, not a relative one.  This takes the deposit off the FP64
+// pipe: 36 of about 165 FP64 instructions per particle for linear shapes.
 __device__ __forceinline__ void emit(double* p, const Amp& a, q62 T) {
-    const u64 jm = mulhi(a.m, (u64)T);  // value jm 2^(e + 2)
-    if (jm != 0ull) red_f64(p, pack_double<false>(jm, a.es + (1087u << 20)));
+    double v;
+    if (contribution(a, T, v)) red_f64(p, v);
 }
 // amplitudes whose contributions may leave the normal doubles: f, the product
 // of the FP64 factors, times the weight
@@ -1053,10 +1052,9 @@ __device__ __forceinline__ void deposit_current(double* J, const Amp& cw, const 
             AccQ s;
             s.mac(Au[j], ak);
             s.mac(Du[j], dk);
-            const q62 T = max(s.get(), 0ll);
             double* row = J + k * sv + j * su;
 #pragma unroll
-            for (int l = 0; l < WP - 1; ++l) emit(row + l * sp, pf[l], T);
+            for (int l = 0; l < WP - 1; ++l) emit(row + l * sp, pf[l], s.get());
         }
     }
 }
@@ -1130,7 +1128,7 @@ __device__ __forceinline__ void deposit_one_axis(int lo, const JView& V, const A
                 AccQ s;
                 s.mac(limb_of(wa.A[i]), ak);
                 s.mac(limb_of(wa.D[i]), dk);
-                emit(J0 + V.cs + k * sb + i * sa, cv, max(s.get(), 0ll));
+                emit(J0 + V.cs + k * sb + i * sa, cv, s.get());
             }
         }
     }
@@ -1159,7 +1157,7 @@ __device__ __forceinline__ bool deposit_q(int lo, const JView& V, const Amp* ja,
     if (DIM == 3) origin += (w1.base + lo) * V.sy;
     const Amp q = amp_of(qw);
     auto out = [&](double* p, const Amp& a, q62 T, double f) {
-        if constexpr (ANY) emit_any(p, f, T);
+        if constexpr (ANY) emit_any(p, f, max(T, 0ll));
         else emit(p, a, T);
     };
     if constexpr (DIM == 3) {
@@ -1200,7 +1198,7 @@ __device__ __forceinline__ bool deposit_q(int lo, const JView& V, const Amp* ja,
                     AccQ s;
                     s.mac(Ab[j], ak);
                     s.mac(Db[j], dk);
-                    const q62 T = max(s.get(), 0ll);
+                    const q62 T = s.get();
                     double* row = plane + j * sb;
 #pragma unroll UW
                     for (int l = 0; l < W - 1; ++l) out(row + l * sa, pf[l], T, nf[l]);
@@ -1236,7 +1234,7 @@ __device__ __forceinline__ bool deposit_q(int lo, const JView& V, const Amp* ja,
                 AccQ s;
                 s.mac(limb_of(w0.A[i]), ak);
                 s.mac(limb_of(w0.D[i]), dk);
-                out(Jy + k * V.sz + i, cv, max(s.get(), 0ll), nfy);
+                out(Jy + k * V.sz + i, cv, s.get(), nfy);
             }
         }
     }
@@ -1259,9 +1257,9 @@ __device__ __forceinline__ bool amps_safe(const ExpRange& r, double qw, double v
 // Linear shapes, particle keeping its cell: the window is the two nodes of the
 // cell, D = (-d, d), one prefix sum, and with the mid-path offsets m and
 // P = m_b m_c + d_b d_c / 12 the four weights are P, m_b - P, m_c - P and
-// 1 - m_b - m_c + P.  cw: prefactor x q w per current (2D: x v_y for y).  P
-// comes out up to 5 units of 2^-62 low: it is raised by 6 and m_b, m_c (by a
-// half low themselves) by 8, so that no weight is negative.
+// 1 - m_b - m_c + P (exactly zero where they should be: a particle on a node and
+// moving along no other direction gives its other nodes nothing).  cw: prefactor x
+// q w per current (2D: x v_y for y).
 template <int DIM>
 __device__ __forceinline__ void deposit_lin_q(int lo, const JView& V, const Amp* cw, const SupQ<1>* n,
                                               const SupQ<1>* mv) {
@@ -1271,9 +1269,8 @@ __device__ __forceinline__ void deposit_lin_q(int lo, const JView& V, const Amp*
     for (int a = 0; a < 3; ++a) {
         if (DIM == 2 && a == 1) continue;
         d[a] = mv[a].w[1] - n[a].w[1];
-        const q62 h = (n[a].w[1] + mv[a].w[1]) >> 1;
-        m[a] = h + 8;
-        lm[a] = limb_of(h);
+        m[a] = (n[a].w[1] + mv[a].w[1]) >> 1;
+        lm[a] = limb_of(m[a]);
         ld[a] = limb_of(d[a]);
         if (a > 0) l12[a] = limb_of(mulq(ld[a], limb_of(kTwelfthQ)));
     }
@@ -1284,8 +1281,8 @@ __device__ __forceinline__ void deposit_lin_q(int lo, const JView& V, const Amp*
         AccQ s;
         s.mac(lb, lc);
         s.mac(db, dc12);
-        const q62 P = s.get() + 6;
-        emit(r, pf, kOneQ + 16 - mb - mc + P);
+        const q62 P = s.get();
+        emit(r, pf, kOneQ - mb - mc + P);
         emit(r + sb, pf, mb - P);
         emit(r + sc, pf, mc - P);
         emit(r + sb + sc, pf, P);
@@ -1301,9 +1298,9 @@ __device__ __forceinline__ void deposit_lin_q(int lo, const JView& V, const Amp*
         }
     } else {
         const Amp px = amp_scale(cw[0], -d[0]), pz = amp_scale(cw[2], -d[2]);
-        emit(origin, px, kOneQ + 8 - m[2]);
+        emit(origin, px, kOneQ - m[2]);
         emit(origin + V.sz, px, m[2]);
-        emit(origin + 2 * V.cs, pz, kOneQ + 8 - m[0]);
+        emit(origin + 2 * V.cs, pz, kOneQ - m[0]);
         emit(origin + 2 * V.cs + 1, pz, m[0]);
         four(origin + V.cs, cw[1], m[0], m[2], lm[0], lm[2], ld[0], l12[2], 1, V.sz);
     }
