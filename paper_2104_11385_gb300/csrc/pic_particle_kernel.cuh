@@ -427,19 +427,22 @@ static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, doubl
     }
 }
 
-// Marks the cells of a staged tile where a component is gathered in FP64: bits +
-// c * words, one bit per tile element.  Every 2 x 2 x 2 nodes of a component (a
-// single node along the half-node directions of the energy-conserving linear
-// gather) must reach weak_limit or be all zero; if not, the cells whose particles
-// interpolate from them are marked: the one at their lower corner, and along a
-// half-node direction the next one too.  (Quadratic shapes: the cell of nearest
-// node.  All orders have those nodes in their particles' supports.)  Linear shapes look at 4 of
-// the 8 nodes, the others, whose limit is higher, at all.  Elements are taken in a
-// row across row ends (what that marks needlessly lies in the halo), 31 windows
-// per warp and round, the components side by side: the shuffle gives the nodes one
-// further in x.  About 1 us per staged tile and CTA (16^3 plasma 40.0 -> 41.2 us
-// per step, 128^3 foil 1365 -> 1393 with the test of the marks, quadratic
-// log-normal boxes 4505 -> 4633).
+// Marks where a component of a staged tile is gathered in FP64: one bit of bits + c
+// * words for each window of 2 x 2 x 2 nodes (a single node along the half-node
+// directions of the energy-conserving linear gather), numbered by the element i of
+// its lower corner (mark_bit), set if it does not reach weak_limit and is not all
+// zero.  A particle looks at the window in the middle of its support
+// (weak_components).  Of a window the two nodes at the lower corner along x are
+// looked at, and the two across from them in y and z: a wave that crosses zero has
+// one of them off the crossing, random noise marks hardly a window.  Elements are
+// taken in a row across row ends, where windows belong to no particle.  A lane
+// takes two windows from two 16-byte loads: shared loads are what this costs,
+// waiting behind the other CTA's reductions.  1 to 5 us per staged tile (16^3
+// plasma 40.7 -> 41.9 us per step, 128^3 foil 1402 -> 1415; one window per 4-byte
+// load 1420).  Without a pass of its own, from the loads that find the largest
+// magnitude, the windows waiting in registers: 1463 (spills).
+__device__ __forceinline__ int mark_word(int i) { return ((i >> 6) << 1) | (i & 1); }
+__device__ __forceinline__ int mark_bit(int i) { return (i >> 1) & 31; }
 template <int ORDER, int DIM>
 __device__ __forceinline__ bool mark_weak(unsigned* __restrict__ bits, int words, const double* __restrict__ sEB,
                                           int stride, int vol, int SX, int SY, const int* __restrict__ emax, bool ec) {
@@ -448,46 +451,53 @@ __device__ __forceinline__ bool mark_weak(unsigned* __restrict__ bits, int words
     unsigned lim[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) lim[c] = emax[c] == 0 ? 0u : weak_limit<ORDER>(emax[c]);
-    const int n = vol - SZ - (DIM == 3 ? SX : 0);  // windows that lie in the tile
-    bool any = false;
-    for (int i0 = (threadIdx.x >> 5) * 31; i0 < n; i0 += (blockDim.x >> 5) * 31) {
-        const int i = min(i0 + lane, n - 1);
-        unsigned weak = 0u;
+    const int n = vol - 2 - SZ - (DIM == 3 ? SX : 0);  // last pair of windows that lie in the tile
+    unsigned any = 0u;
+    for (int w = 2 * (threadIdx.x >> 5); w < words; w += 2 * (blockDim.x >> 5)) {
+        const int i = min(32 * w + 2 * lane, n);  // (n is even: rows have even lengths)
+        uint2 mine = make_uint2(0u, 0u);
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
             const int a = c < 3 ? c : c - 3;
             const bool isb = c >= 3, hx = (a == 0) != isb, hy = (a == 1) != isb, hz = (a == 2) != isb;
-            const int dy = DIM == 2 || (one && hy) ? 0 : SX, dz = one && hz ? 0 : SZ;
-            const unsigned* h = reinterpret_cast<const unsigned*>(sEB + c * stride) + 1;  // high words
-            auto mag = [&](int k) { return h[2 * k] & 0x7FFFFFFFu; };
-            unsigned m = max(mag(i), mag(i + dy + dz));
-            if (DIM == 3 && (ORDER > 1 || one)) m = max(m, max(mag(i + dy), mag(i + dz)));
-            const unsigned mx = __shfl_down_sync(0xffffffffu, m, 1);
-            if (!(one && hx)) m = max(m, mx);
-            weak |= m != 0u && m < lim[c] ? 1u << c : 0u;
-        }
-        if (lane == 31 || i0 + lane >= n) weak = 0u;
-        if (__any_sync(0xffffffffu, weak != 0u)) {
-            any = true;
-#pragma unroll 1
-            for (int c = 0; c < 6; ++c) {
-                const unsigned w = __ballot_sync(0xffffffffu, (weak >> c) & 1u);
-                if (w == 0u) continue;
-                const int a = c < 3 ? c : c - 3;
-                const bool isb = c >= 3, hx = (a == 0) != isb, hy = DIM == 3 && ((a == 1) != isb), hz = (a == 2) != isb;
-                // lane: along which of the half-node directions the marked cell is the next one
-                if (lane < 8 && (!(lane & 1) || (hx && !one)) && (!(lane & 2) || (hy && !one)) &&
-                    (!(lane & 4) || (hz && !one))) {
-                    const int b = i0 + (lane & 1 ? 1 : 0) + (lane & 2 ? SX : 0) + (lane & 4 ? SZ : 0);
-                    const unsigned up = (b & 31) ? w >> (32 - (b & 31)) : 0u;
-                    unsigned* const to = bits + c * words + (b >> 5);
-                    if ((b >> 5) < words) atomicOr(to, w << (b & 31));
-                    if (up != 0u && (b >> 5) + 1 < words) atomicOr(to + 1, up);
-                }
+            const int d = (DIM == 2 || (one && hy) ? 0 : SX) + (one && hz ? 0 : SZ);
+            const uint4 v = *reinterpret_cast<const uint4*>(sEB + c * stride + i);
+            const uint4 u = *reinterpret_cast<const uint4*>(sEB + c * stride + i + d);
+            unsigned m0 = max(v.y & 0x7FFFFFFFu, u.y & 0x7FFFFFFFu);  // (high words)
+            unsigned m1 = max(v.w & 0x7FFFFFFFu, u.w & 0x7FFFFFFFu);
+            const unsigned next = __shfl_down_sync(0xffffffffu, m0, 1);
+            if (!(one && hx)) {
+                m0 = max(m0, m1);
+                m1 = lane == 31 ? m1 : max(m1, next);
             }
+            const unsigned w0 = __ballot_sync(0xffffffffu, m0 != 0u && m0 < lim[c]);
+            const unsigned w1 = __ballot_sync(0xffffffffu, m1 != 0u && m1 < lim[c]);
+            any |= w0 | w1;
+            if (lane == c) mine = make_uint2(w0, w1);
         }
+        if (lane < 6) *reinterpret_cast<uint2*>(bits + lane * words + w) = mine;
     }
-    return any;
+    return any != 0u;
+}
+// the components (bits) that a particle gathers in FP64, from its supports and the marks
+template <int ORDER, int DIM>
+__device__ __forceinline__ unsigned weak_components(const unsigned* __restrict__ bits, int words, int SX, int SY,
+                                                    const SupQ<ORDER>* nd, const AxisQ<ORDER>* hf) {
+    // lower node of the window along an axis: for quadratic shapes those at the
+    // nearest node and half a cell below it lie in every support
+    constexpr int H = EBHalo<ORDER>::lo, BN = H + (ORDER == 1 ? 0 : 1), BH = H + (ORDER == 3 ? 1 : 0);
+    auto half = [&](int a) { return (ORDER == 2 ? nd[a].s : hf[a].s) + BH; };
+    const int SZ = SX * SY, nx = nd[0].s + BN, hx = half(0), nz = (nd[2].s + BN) * SZ, hz = half(2) * SZ;
+    const int ny = DIM == 3 ? (nd[1].s + BN) * SX : 0, hy = DIM == 3 ? half(1) * SX : 0;
+    unsigned mask = 0u;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const int a = c < 3 ? c : c - 3;
+        const bool isb = c >= 3;
+        const int i = ((a == 0) != isb ? hx : nx) + ((a == 1) != isb ? hy : ny) + ((a == 2) != isb ? hz : nz);
+        mask |= ((bits[c * words + mark_word(i)] >> mark_bit(i)) & 1u) << c;
+    }
+    return mask;
 }
 
 // Esirkepov node shapes on a common window of W nodes starting at the lower of
@@ -697,7 +707,7 @@ __host__ __device__ inline SmemPlan smem_plan(const int ebs[3]) {
     p.pb_off = 6 * p.eb_stride;
     // tiles too large to leave room for the buffers (2D tiles of 64 cells) load
     // their particles directly
-    p.bit_words = (p.eb_vol + 31) / 32;
+    p.bit_words = 2 * ((p.eb_vol + 63) / 64);
     const int bits = 3 * p.bit_words;  // doubles that 6 components' words take
     p.staged = (p.pb_off + PIC_PBUF_DOUBLES + bits) * sizeof(double) <= 225 * 1024;
     p.bit_off = p.pb_off + (p.staged ? PIC_PBUF_DOUBLES : 0);
@@ -1381,7 +1391,7 @@ __device__ __forceinline__ PIn read_staged(const double* slot) {
 // weak: its cells where a component is gathered in FP64, nullptr if there is none.
 template <class R, int DIM, int ORDER, class SV, class SPV>
 __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const SimDev& SG, const Tile& tl,
-                                           const double* __restrict__ sEB, const unsigned* weak,
+                                           const double* __restrict__ sEB, const unsigned* __restrict__ weak,
                                            const int* __restrict__ emax,
                                            const JView& V, double* __restrict__ sQw, unsigned* s_one, unsigned* s_many,
                                            const SmemPlan& P, const R* dtd, R kq, double qs, int64_t p, const PIn& in,
@@ -1415,13 +1425,10 @@ __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const Sim
         }
         f = gather6_q<ORDER, DIM>(reinterpret_cast<const long long*>(sEB), P.eb_stride, S.ebs[0], S.ebs[1], emax, na, ha);
         if (weak) {
-            // the particle's cell (quadratic: its nearest node)
-            constexpr int B = EBHalo<ORDER>::lo + (ORDER == 1 ? 0 : 1);
-            const int i = ((nd[2].s + B) * S.ebs[1] + (DIM == 3 ? nd[1].s + B : 0)) * S.ebs[0] + nd[0].s + B;
-            weak += i >> 5;
-#pragma unroll 1
-            for (int c = 0; c < 6; ++c, weak += P.bit_words) {
-                if (((*weak >> (i & 31)) & 1u) == 0u) continue;
+            unsigned mask = weak_components<ORDER, DIM>(weak, P.bit_words, S.ebs[0], S.ebs[1], nd, ha);
+            while (mask != 0u) {
+                const int c = __ffs((int)mask) - 1;
+                mask &= mask - 1u;
                 const double v = gather1_fp64<ORDER, DIM>(SG, c, x0[0], x0[1], x0[2], tl.o[0], tl.o[1], tl.o[2]);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) f.v[k] = c == k ? v : f.v[k];
@@ -2116,8 +2123,6 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                         for (int c = 0; c < 6; ++c)
                             tma_load_3d(sEBd + c * P.eb_stride, &S.tmap[c], x0, y0, z0, &bar);
                     }
-                    if (PREC != 2)
-                        for (int i = threadIdx.x; i < 6 * P.bit_words; i += blockDim.x) s_bits[i] = 0u;
                     for (int i = threadIdx.x; i < 9; i += blockDim.x) {
                         const int a = i / 3, side = i - 3 * a;
                         const int c = a == 0 ? cur.o[0] : (a == 1 ? cur.o[1] : cur.o[2]);
