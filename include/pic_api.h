@@ -180,7 +180,11 @@ enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
  *   cap_factor  knapsack cap on units per worker, times the average (1.5).
  *   n_workers   workers the mapping spreads over; 0 = one per persistent CTA.
  *   split       target work units per worker used to cut heavy boxes into
- *               several units (CTAs per box); 0 = library default.
+ *               several units (CTAs per box); 0 = library default.  Units are
+ *               not cut below 1024 to 4096 particles (a quarter of a worker's
+ *               share; in runs too small for that, down to 256 so that every
+ *               worker has one), and below that only where the mapping is
+ *               badly balanced by measured costs.
  *   sched       LISTS: each persistent CTA runs its own worker's units;
  *               QUEUE: all CTAs pull units from one list in mapping order. */
 typedef struct {

@@ -266,17 +266,6 @@ int64_t unit_share(const pic_sim* s, int64_t nu) {
     return std::max<int64_t>(1, std::min<int64_t>(s->ctas / nu, np / nu / 256));
 }
 
-// Particles below which a heavy box is not cut further.  A unit costs about 14
-// us of scheduling, tile staging and partly filled rounds before any balance is
-// gained (128^3 foil, 8.4 M particles on 304 CTAs: 1.48 ms in units of 1725
-// particles, 1.31 ms in units of 6900), so units hold at least 4096 particles,
-// or a quarter of a worker's share where that is less, and never below 1024.
-int64_t min_unit_particles(const std::vector<int64_t>& np, int n_workers) {
-    int64_t total = 0;
-    for (int64_t n : np) total += n;
-    return std::max<int64_t>(1024, std::min<int64_t>(4096, total / (4 * std::max(1, n_workers))));
-}
-
 pic_status upload_plan(pic_sim* s) {
     const SimPlan& P = s->plan;
     std::vector<UnitDev> units = P.units;
@@ -436,6 +425,38 @@ void map_units(const pic_sim* s, const pic_lb_params& p, const std::vector<pic::
     }
 }
 
+// Cuts the boxes into units and maps them.  Where that balances badly by measured
+// costs (E < 0.8: few units, and particles of unequal cost), finer cuts are tried
+// too, and the one whose heaviest worker ends first is taken, every unit counted
+// with the 14 us a step that it costs by itself.  Foil of 64 x 96 x 64 cells and 393
+// thousand particles after the pulse has hit it: particle kernel 573 -> 516 us.
+void cut_and_map(const pic_sim* s, const pic_lb_params& p, const std::vector<double>& costs, const std::vector<int64_t>& np,
+                 int64_t steps, int nw, std::vector<pic::Unit>& units, std::vector<double>& uc, std::vector<int32_t>& assign) {
+    const int64_t nb = s->h.nboxes;
+    const int split = p.split > 0 ? p.split : s->split;
+    int64_t least = pic::min_unit_particles(np.data(), nb, nw);
+    units = pic::make_units(costs.data(), np.data(), nb, nw, split, least, true);
+    map_units(s, p, units, nw, uc, assign);
+    if (p.cost == PIC_COST_HEURISTIC || p.policy == PIC_POLICY_BOX_ORDER || steps <= 0 ||
+        pic::lb_efficiency(uc.data(), assign.data(), (int64_t)uc.size(), nw) >= 0.8)
+        return;
+    const double unit_us = 14.0;  // in ns, or in clocks of a CTA's threads at 2 GHz
+    const double ov = (double)steps * unit_us * (p.cost == PIC_COST_KERNEL_TIME ? 1e3 : 2e3 * s->threads);
+    double best = pic::makespan(uc.data(), assign.data(), (int64_t)uc.size(), nw, ov);
+    while ((least /= 2) >= 256) {
+        std::vector<pic::Unit> u2 = pic::make_units(costs.data(), np.data(), nb, nw, split, least, true);
+        std::vector<double> c2;
+        std::vector<int32_t> a2;
+        map_units(s, p, u2, nw, c2, a2);
+        const double t = pic::makespan(c2.data(), a2.data(), (int64_t)c2.size(), nw, ov);
+        if (t >= best) continue;
+        best = t;
+        units.swap(u2);
+        uc.swap(c2);
+        assign.swap(a2);
+    }
+}
+
 pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_result* out) {
     std::vector<double> costs;
     std::vector<int64_t> np;
@@ -444,12 +465,10 @@ pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_re
     const int nw = n_workers_for(s, p);
     // E_old: the mapping in force, re-costed with the costs just measured
     const double e_old = plan_efficiency(s, costs);
-    const int split = p.split > 0 ? p.split : s->split;
-    std::vector<pic::Unit> units =
-        pic::make_units(costs.data(), np.data(), nb, nw, split, min_unit_particles(np, nw), true);
+    std::vector<pic::Unit> units;
     std::vector<double> uc;
     std::vector<int32_t> assign;
-    map_units(s, p, units, nw, uc, assign);
+    cut_and_map(s, p, costs, np, s->cost_steps, nw, units, uc, assign);
     double e_new = pic::lb_efficiency(uc.data(), assign.data(), (int64_t)uc.size(), nw);
     bool adopted = pic::adopt(e_old, e_new, theta);
     if (adopted) {
@@ -458,6 +477,8 @@ pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_re
     }
     s->last_costs = costs;
     s->last_np = np;
+    s->last_steps = s->cost_steps;
+    s->cost_steps = 0;
     CU(s, cudaMemsetAsync(s->h.cost_clock, 0, nb * sizeof(uint64_t), s->stream));
     CU(s, cudaMemsetAsync(s->h.cost_time, 0, nb * sizeof(uint64_t), s->stream));
     pic_lb_result r;
@@ -628,12 +649,10 @@ pic_status replan(pic_sim* s) {
     pic_lb_params p = s->lb_set ? s->lb : default_lb();
     if (p.mode == PIC_LB_NONE || s->last_costs.empty()) return initial_plan(s);
     const int nw = n_workers_for(s, p);
-    const int split = p.split > 0 ? p.split : s->split;
-    std::vector<pic::Unit> units = pic::make_units(s->last_costs.data(), s->last_np.data(),
-                                                   s->h.nboxes, nw, split, min_unit_particles(s->last_np, nw), true);
+    std::vector<pic::Unit> units;
     std::vector<double> uc;
     std::vector<int32_t> assign;
-    map_units(s, p, units, nw, uc, assign);  // the simulation's own policy
+    cut_and_map(s, p, s->last_costs, s->last_np, s->last_steps, nw, units, uc, assign);  // the simulation's own policy
     build_plan(s, units, assign, nw, p.sched, p.policy == PIC_POLICY_BOX_ORDER);
     return upload_plan(s);
 }
@@ -1090,6 +1109,7 @@ pic_status pic_step(pic_sim* s, int nsteps) {
         st.launches += s->kernels_per_step ? s->kernels_per_step : count_kernels(s);
         st.particle_launches += s->h.nsp > 0 ? 1 : 0;
         s->step_count++;
+        s->cost_steps++;
         const pic_lb_params& p = s->lb;
         if (s->lb_set && p.mode != PIC_LB_NONE && s->step_count % p.interval == 0) {
             if (p.mode == PIC_LB_DYNAMIC) {
@@ -1159,6 +1179,7 @@ pic_status pic_get_efficiency(pic_sim* s, int strategy, int reset_window, double
     if (reset_window) {
         CU(s, cudaMemsetAsync(s->h.cost_clock, 0, s->h.nboxes * sizeof(uint64_t), s->stream));
         CU(s, cudaMemsetAsync(s->h.cost_time, 0, s->h.nboxes * sizeof(uint64_t), s->stream));
+        s->cost_steps = 0;
         CU(s, cudaStreamSynchronize(s->stream));
     }
     return PIC_OK;

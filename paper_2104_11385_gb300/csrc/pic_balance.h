@@ -28,4 +28,9 @@ struct Unit {
 std::vector<Unit> make_units(const double* costs, const int64_t* np, int64_t nboxes, int n_workers,
                              int split, int64_t min_particles, bool allow_split);
 
+// particles below which a box is not cut further (make_units' min_particles)
+int64_t min_unit_particles(const int64_t* np, int64_t nboxes, int n_workers);
+// the heaviest worker's load when every unit costs `overhead` on top of its own
+double makespan(const double* costs, const int32_t* assign, int64_t nunits, int n_workers, double overhead);
+
 }  // namespace pic

@@ -1,0 +1,33 @@
+"""Small runs under a scheduler: enough work units for every persistent CTA."""
+import pytest
+import torch
+
+import paper_2104_11385_gb300 as pic
+from paper_2104_11385_gb300 import workloads
+from test_gpu_parity import compare, make_gpu, make_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("npart", [40000, 130000, 300000])
+@pytest.mark.parametrize("sched", [pic.SCHED_QUEUE, pic.SCHED_LISTS])
+def test_heavy_boxes_are_cut_for_all_ctas(npart, sched):
+    """16 boxes hold every particle; the cut leaves no unit below 256 particles and,
+    where there are 256 per CTA, a unit for at least three CTAs of four"""
+    wl = workloads.random_plasma(73, 3, (32, 32, 64), (16, 16, 16), (0.3, 0.3, 0.3), 1, nspecies=1, npart=npart, umax=0.5)
+    sp = wl["species"][0]
+    sp["z"] *= 0.249  # into the first layer of boxes, 4 of 16
+    sim = make_gpu(wl)
+    ctas = sim.get_launch()["ctas_per_sm"] * torch.cuda.get_device_properties(0).multi_processor_count
+    r = sim.rebalance(mode=pic.LB_DYNAMIC, interval=10, theta=0.0, cost=pic.COST_HEURISTIC, sched=sched)
+    with_particles = r["n_units"] - 12
+    assert with_particles <= max(4, npart // 256)
+    if npart >= 256 * ctas:
+        assert with_particles >= 0.75 * ctas
+    else:
+        assert with_particles >= 0.75 * npart / 256
+    if npart == 40000:
+        ref = make_oracle(wl)
+        sim.step(3)
+        ref.step(3)
+        compare(sim, ref, wl)
