@@ -71,8 +71,7 @@ __global__ void bin_count_kernel(BinGeom g, const double* __restrict__ x, const 
 }
 
 // The same through a histogram in shared memory per CTA, added to the global one
-// at the end: for many particles per box (bin_shared).
-constexpr int kBinHistMax = 8192;  // boxes: 32 KB
+// at the end: for many particles per box (bin_count_in_shared).
 __global__ void __launch_bounds__(1024) bin_count_shared_kernel(BinGeom g, const double* __restrict__ x,
                                                                 const double* __restrict__ y,
                                                                 const double* __restrict__ z, int64_t np,
@@ -130,12 +129,12 @@ __global__ void bin_scatter_kernel(BinGeom g, const double* __restrict__ x, cons
     }
 }
 
-// The scatter for the same inputs: a CTA ranks 16 positions per thread in shared
-// memory and takes one global cursor step per box it met instead of one per
-// position (a returning atomic each, contended where boxes are few).  Per call:
+// The scatter of large inputs (bin_scatter_in_shared): a CTA ranks 16 positions
+// per thread in shared memory and takes one global cursor step per box it met
+// instead of one per position (a returning atomic each, contended where boxes are
+// few).  Per call:
 // 1 M positions in 512 boxes 156 -> 57 us, 16.8 M in 4096 boxes 704 -> 589 us
 // shuffled and 857 -> 534 ordered along z.
-constexpr int kBinPer = 16;
 __global__ void __launch_bounds__(1024) bin_scatter_shared_kernel(BinGeom g, const double* __restrict__ x,
                                                                   const double* __restrict__ y,
                                                                   const double* __restrict__ z, int64_t np,
@@ -168,11 +167,6 @@ __global__ void __launch_bounds__(1024) bin_scatter_shared_kernel(BinGeom g, con
         __syncthreads();
     }
 }
-
-// the shared histograms pay when adding them up takes at most a quarter of the
-// global atomics they save (counts of 16.8 M positions in 4096 boxes: 803 -> 704
-// us per call; 100 thousand positions there stay with the global ones, 31 us)
-bool bin_shared(int nboxes, int64_t np, int ctas) { return nboxes <= kBinHistMax && np >= 4ll * ctas * nboxes; }
 
 int bin_grid(int64_t np) {
     int64_t b = (np + 255) / 256;
@@ -231,12 +225,12 @@ cudaError_t pic_bin_launch(const BinGeom& g, const double* x, const double* y, c
     if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, (size_t)g.nboxes * sizeof(int32_t), st);
     if (e != cudaSuccess) return e;
     const int wide = 2 * pic_sm_count();  // CTAs of 1024 threads, two per SM
-    if (np > 0 && bin_shared(g.nboxes, np, wide))
+    if (np > 0 && bin_count_in_shared(g.nboxes, np, wide))
         bin_count_shared_kernel<<<wide, 1024, 0, st>>>(g, x, y, z, np, (unsigned long long*)box_off);
     else if (np > 0)
         bin_count_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, (unsigned long long*)box_off);
     bin_scan_kernel<<<1, 1024, 0, st>>>(box_off, g.nboxes);
-    if (np > 0 && bin_shared(g.nboxes, np, wide))
+    if (np > 0 && bin_scatter_in_shared(g.nboxes, np, wide))
         bin_scatter_shared_kernel<<<wide, 1024, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
     else if (np > 0)
         bin_scatter_kernel<<<bin_grid(np), 256, 0, st>>>(g, x, y, z, np, box_off, cursor, perm);
