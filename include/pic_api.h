@@ -175,6 +175,11 @@ enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
  *               %globaltimer span of the box's particle loops, the mean over
  *               each CTA's warps: the in-kernel
  *               analog of the paper's CUPTI kernel duration, without CUPTI).
+ *               The mean, because a unit that leaves warps idle is charged for
+ *               the share it uses; the loops alone, because the tile staging
+ *               before them takes about as long for every small box and would
+ *               hide how their work differs.  It is a fixed cost per unit, and
+ *               counted as one (14 us) where cuts into units are compared.
  *   w_p, w_c    heuristic weights (Sec. 3.3 footnotes: 0.75/0.25 knapsack,
  *               0.02/0.98 SFC).
  *   cap_factor  knapsack cap on units per worker, times the average (1.5).
