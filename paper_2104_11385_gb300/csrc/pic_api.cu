@@ -253,17 +253,14 @@ void build_plan(pic_sim* s, const std::vector<pic::Unit>& units, const std::vect
     }
 }
 
-// CTAs that share one work unit.  A mapping with at most half as many units as
-// persistent CTAs (8 boxes on 152 SMs) would leave most of the chip idle, so
-// each unit is then cut into equal parts that different CTAs pull, down to 256
-// particles (one round of a CTA's threads).  The plan itself, its costs and its
-// efficiency stay per unit.  16^3 cells in 8 boxes, 32768 particles, one CTA per
-// SM: the particle kernel takes 40 us against 137.
-int64_t unit_share(const pic_sim* s, int64_t nu) {
-    if (nu == 0 || 2 * nu > s->ctas) return 1;
-    int64_t np = 0;
-    for (int i = 0; i < s->h.nsp; ++i) np += s->np_init[i];
-    return std::max<int64_t>(1, std::min<int64_t>(s->ctas / nu, np / nu / 256));
+pic_status box_counts(pic_sim* s, std::vector<int64_t>& np) {
+    np.assign(s->h.nboxes, 0);
+    if (s->h.nsp == 0) return PIC_OK;
+    CU(s, pic_launch_box_counts(s->d, s->h, s->d_box_np, s->stream));
+    CU(s, cudaMemcpyAsync(np.data(), s->d_box_np, s->h.nboxes * sizeof(int64_t),
+                          cudaMemcpyDeviceToHost, s->stream));
+    CU(s, cudaStreamSynchronize(s->stream));
+    return PIC_OK;
 }
 
 pic_status upload_plan(pic_sim* s) {
@@ -271,7 +268,13 @@ pic_status upload_plan(pic_sim* s) {
     std::vector<UnitDev> units = P.units;
     std::vector<int32_t> list_off = P.list_off;
     int nlists = P.nlists;
-    const int64_t share = unit_share(s, (int64_t)units.size());
+    int64_t np = 0;
+    if (2 * (int64_t)units.size() <= s->ctas) {  // (few units: how many particles there are now)
+        std::vector<int64_t> now;
+        TRY(box_counts(s, now));
+        for (int64_t n : now) np += n;
+    }
+    const int64_t share = pic::unit_share((int64_t)units.size(), s->ctas, np);
     if (share > 1) {
         units.clear();
         for (const UnitDev& u : P.units)
@@ -338,16 +341,6 @@ pic_status initial_plan(pic_sim* s) {
 }
 
 // ---------------------------------------------------------------- costs ---
-pic_status box_counts(pic_sim* s, std::vector<int64_t>& np) {
-    np.assign(s->h.nboxes, 0);
-    if (s->h.nsp == 0) return PIC_OK;
-    CU(s, pic_launch_box_counts(s->d, s->h, s->d_box_np, s->stream));
-    CU(s, cudaMemcpyAsync(np.data(), s->d_box_np, s->h.nboxes * sizeof(int64_t),
-                          cudaMemcpyDeviceToHost, s->stream));
-    CU(s, cudaStreamSynchronize(s->stream));
-    return PIC_OK;
-}
-
 pic_status box_costs(pic_sim* s, int strategy, double w_p, double w_c, std::vector<double>& costs,
                      std::vector<int64_t>& np) {
     TRY(box_counts(s, np));

@@ -155,6 +155,17 @@ int64_t min_unit_particles(const int64_t* np, int64_t nboxes, int n_workers) {
     return hi;
 }
 
+// A mapping with at most half as many units as persistent CTAs (8 boxes on 152
+// SMs) would leave most of the chip idle, so each unit is then cut into equal
+// parts that different CTAs pull, down to 256 particles (one round of a CTA's
+// threads).  The plan itself, its costs and its efficiency stay per unit.  16^3
+// cells in 8 boxes, 32768 particles, one CTA per SM: the particle kernel takes 40
+// us against 137.
+int64_t unit_share(int64_t nu, int ctas, int64_t np) {
+    if (nu <= 0 || 2 * nu > ctas) return 1;
+    return std::max<int64_t>(1, std::min<int64_t>(ctas / nu, np / nu / 256));
+}
+
 double makespan(const double* costs, const int32_t* assign, int64_t nunits, int n_workers, double overhead) {
     std::vector<double> load(n_workers, 0.0);
     double mx = 0.0;

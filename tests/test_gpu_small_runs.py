@@ -1,4 +1,5 @@
 """Small runs under a scheduler: enough work units for every persistent CTA."""
+import numpy as np
 import pytest
 import torch
 
@@ -31,3 +32,20 @@ def test_heavy_boxes_are_cut_for_all_ctas(npart, sched):
         sim.step(3)
         ref.step(3)
         compare(sim, ref, wl)
+
+
+@pytest.mark.parametrize("sched", [pic.SCHED_QUEUE, pic.SCHED_LISTS])
+def test_units_after_most_particles_left(sched):
+    """few boxes, nearly all particles absorbed: a mapping made then is cut for what is left"""
+    wl = workloads.random_plasma(75, 3, (16, 16, 32), (8, 8, 16), (0.3, 0.3, 0.3), 1, nspecies=1, npart=20000, umax=0.5,
+                                 absorb=6)
+    sp = wl["species"][0]
+    sp["uz"][:19000] = np.where(sp["z"][:19000] < 4.8, -50.0, 50.0)  # out through the nearer layer
+    sim, ref = make_gpu(wl), make_oracle(wl)
+    for s in (sim, ref):
+        s.step(24)
+    assert sim.num_particles(0) < 5000
+    sim.rebalance(mode=pic.LB_DYNAMIC, interval=10, theta=0.0, cost=pic.COST_HEURISTIC, sched=sched)
+    for s in (sim, ref):
+        s.step(3)
+    compare(sim, ref, wl)

@@ -11,6 +11,7 @@ SHIM = r"""
 #include "pic_balance.cpp"
 extern "C" {
 int64_t t_min(const int64_t* np, int64_t nb, int nw) { return pic::min_unit_particles(np, nb, nw); }
+int64_t t_share(int64_t nu, int ctas, int64_t np) { return pic::unit_share(nu, ctas, np); }
 double t_span(const double* c, const int32_t* a, int64_t n, int nw, double o) { return pic::makespan(c, a, n, nw, o); }
 }
 """
@@ -24,7 +25,7 @@ def lib(tmp_path_factory):
     csrc = os.path.join(ROOT, "paper_2104_11385_gb300", "csrc")
     subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", csrc, str(d / "shim.cpp"), "-o", str(so)])
     L = ctypes.CDLL(str(so))
-    L.t_min.restype = ctypes.c_int64
+    L.t_min.restype = L.t_share.restype = ctypes.c_int64
     L.t_span.restype = ctypes.c_double
     return L
 
@@ -69,3 +70,9 @@ def test_makespan(lib):
     f = lambda o: lib.t_span(c.ctypes.data_as(ctypes.c_void_p), a.ctypes.data_as(ctypes.c_void_p), ctypes.c_int64(4), 3,
                              ctypes.c_double(o))
     assert f(0.0) == 5.0 and f(1.0) == 6.0 and f(4.0) == 10.0
+
+
+@pytest.mark.parametrize("nu,ctas,np_,want", [(8, 152, 32768, 16), (8, 152, 400, 1), (8, 152, 0, 1), (76, 152, 10 ** 6, 2),
+                                              (77, 152, 10 ** 6, 1), (1, 304, 10 ** 6, 304), (0, 304, 10, 1)])
+def test_share(lib, nu, ctas, np_, want):
+    assert lib.t_share(ctypes.c_int64(nu), ctas, ctypes.c_int64(np_)) == want
