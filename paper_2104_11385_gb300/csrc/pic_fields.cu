@@ -103,6 +103,11 @@ __device__ __noinline__ double antenna_amp(const SimDev& S) {
     return 2.0 * L.a0 / S.d[2] * exp(-tt * tt) * sin(L.omega * (t - L.t_peak));
 }
 
+// (one warp; a field sub-step's own launch)
+__global__ void antenna_kernel(SimDev* __restrict__ sims) {
+    if (threadIdx.x == 0) sims[0].las.amp = antenna_amp(sims[0]);
+}
+
 // B half step.  A step's first one also folds the current (nfold further
 // blocks: the two touch different arrays, and share one launch) and leaves the
 // antenna's time factor for the E step (in one thread: FP64 exp and sin are
@@ -341,13 +346,16 @@ cudaError_t pic_launch_fold(const SimDev* dsim, const SimDev& h, cudaStream_t st
 cudaError_t pic_launch_field_stage(const SimDev* dsim, const SimDev& h, int stage, cudaStream_t st) {
     const int nb = row_blocks(h);
     if (stage == 0 || stage == 2) {
-        if (h.dim == 3) b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr, stage == 0, 0);
-        else b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr, stage == 0, 0);
+        if (h.dim == 3) b_half_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr, 0, 0);
+        else b_half_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr, 0, 0);
         if (stage == 2 && h.absorb > 0) {
             int64_t t = (int64_t)h.n[0] * h.n[1] * 2 * h.absorb;
             damp_kernel<<<blocks_for(t, 256), 256, 0, st>>>(dsim, nullptr);
         }
     } else if (stage == 1) {
+        // the factor belongs to this sub-step: others may come between it and the
+        // first one, and so may a change of the device copy or of the step number
+        if (h.las.on) antenna_kernel<<<1, 32, 0, st>>>(const_cast<SimDev*>(dsim));
         if (h.dim == 3) e_kernel<3><<<nb, 256, 0, st>>>(dsim, nullptr);
         else e_kernel<2><<<nb, 256, 0, st>>>(dsim, nullptr);
     } else {
