@@ -191,7 +191,11 @@ enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
  *               worker has one), and below that only where the mapping is
  *               badly balanced by measured costs.
  *   sched       LISTS: each persistent CTA runs its own worker's units;
- *               QUEUE: all CTAs pull units from one list in mapping order. */
+ *               QUEUE: all CTAs pull units from one list in mapping order.
+ *               A mapping with at most half as many units as CTAs is run as
+ *               one queue under either, in mapping order, each unit cut into
+ *               equal parts for the idle CTAs; the mapping itself, its costs
+ *               and its efficiency stay those of the uncut units. */
 typedef struct {
     int mode, interval;
     double theta;
@@ -266,6 +270,9 @@ pic_status pic_set_cost_capture(pic_sim* sim, int mask);
  * with the per-box costs of the current cost window (strategy as in
  * pic_get_box_costs; a box's cost is divided evenly over its work units), as
  * Listing 1 evaluates the current distribution before it proposes a new one.
+ * It is the mapping's: where few units are shared by several CTAs (see sched)
+ * E does not count the sharing (8 equal boxes on 152 workers: E = 8/152, though
+ * every CTA has work), and neither do e_old, e_new and the log.
  * The cost window is the one pic_rebalance reads: it holds everything since
  * the last load-balancing call.  reset_window != 0 starts a new window after
  * the read (the next internal load-balancing call then sees only the steps

@@ -49,3 +49,15 @@ def test_units_after_most_particles_left(sched):
     for s in (sim, ref):
         s.step(3)
     compare(sim, ref, wl)
+
+
+@pytest.mark.parametrize("sched", [pic.SCHED_QUEUE, pic.SCHED_LISTS])
+def test_efficiency_of_shared_units_is_the_mappings(sched):
+    """8 boxes shared by all CTAs: E counts the 8 units, one worker each"""
+    wl = workloads.random_plasma(77, 3, (16, 16, 16), (8, 8, 8), (0.3, 0.3, 0.3), 1, nspecies=1, npart=20000, umax=0.5)
+    sim = make_gpu(wl)
+    sim.set_lb_params(mode=pic.LB_DYNAMIC, interval=1000, theta=0.0, cost=pic.COST_HEURISTIC, sched=sched)
+    sim.step(1)
+    costs, _ = sim.box_costs(pic.COST_HEURISTIC)
+    workers = sim.get_launch()["ctas_per_sm"] * torch.cuda.get_device_properties(0).multi_processor_count
+    assert sim.efficiency(pic.COST_HEURISTIC) == pytest.approx(costs.sum() / workers / costs.max(), rel=1e-12)
