@@ -544,7 +544,7 @@ pic_status capture_graph(pic_sim* s) {
 }
 
 pic_status configure_launch(pic_sim* s) {
-    s->smem = pic_particle_smem_bytes(s->h.dim, s->h.order, s->h.T, s->threads, s->prec);
+    s->smem = pic_particle_smem_bytes(s->h.dim, s->h.order, s->h.T);
     cudaDeviceProp prop;
     CU(s, cudaGetDeviceProperties(&prop, s->device));
     if (s->smem > prop.sharedMemPerBlockOptin)
@@ -588,7 +588,7 @@ pic_status retile(pic_sim* s, int t) {
         set_tiling(probe, tt);
         cudaDeviceProp prop;
         CU(s, cudaGetDeviceProperties(&prop, s->device));
-        if (pic_particle_smem_bytes(h.dim, h.order, probe.T, s->threads, s->prec) > prop.sharedMemPerBlockOptin)
+        if (pic_particle_smem_bytes(h.dim, h.order, probe.T) > prop.sharedMemPerBlockOptin)
             return fail(s, PIC_EUNSUPPORTED, "tile %d does not fit in shared memory", t);
     }
     TRY(sync_and_check(s));
@@ -1388,7 +1388,7 @@ pic_status pic_autotune(pic_sim* s, int steps_per_candidate, pic_launch_cfg* bes
         set_tiling(probe, tt);
         cudaDeviceProp prop;
         CU(s, cudaGetDeviceProperties(&prop, s->device));
-        if (pic_particle_smem_bytes(probe.dim, probe.order, probe.T, 256, s->prec) > prop.sharedMemPerBlockOptin)
+        if (pic_particle_smem_bytes(probe.dim, probe.order, probe.T) > prop.sharedMemPerBlockOptin)
             continue;
         for (int ppt = 1; ppt <= 2; ++ppt) {
             pic_launch_cfg c = best_ms < 1e29f ? best_cfg : cur;

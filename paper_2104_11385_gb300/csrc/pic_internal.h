@@ -148,7 +148,7 @@ struct LaunchCfg {
     int ppt = 1;  // particles per thread per loop iteration (1 or 2)
 };
 // dynamic shared memory of the particle kernel (every precision)
-size_t pic_particle_smem_bytes(int dim, int order, const int T[3], int threads, int prec);
+size_t pic_particle_smem_bytes(int dim, int order, const int T[3]);
 cudaError_t pic_prepare_particles(int dim, int order, size_t smem);  // outside graph capture
 int pic_particle_occupancy(int dim, int order, int minb, int ppt, int threads, size_t smem,
                            int prec);  // resident CTAs per SM

@@ -5,7 +5,7 @@
 
 PIC_DEFINE_PARTICLE_TU(p0_d3)
 
-size_t pic_particle_smem_bytes(int dim, int order, const int T[3], int threads, int prec) {
+size_t pic_particle_smem_bytes(int dim, int order, const int T[3]) {
     int ebs[3];
     for (int a = 0; a < 3; ++a) {
         bool act = !(dim == 2 && a == 1);

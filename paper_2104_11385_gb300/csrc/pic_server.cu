@@ -231,7 +231,7 @@ pic_status admit(pic_server* s, Request& r, int slot) {
     s->max_padded = std::max(s->max_padded, pvol);
     s->max_cells = std::max(s->max_cells, (int64_t)mirror.n[0] * mirror.n[1] * mirror.n[2]);
     for (int i = 0; i < mirror.nsp; ++i) s->max_cap = std::max(s->max_cap, mirror.sp[i].cap);
-    s->smem = std::max(s->smem, pic_particle_smem_bytes(mirror.dim, mirror.order, mirror.T, s->threads, 0));
+    s->smem = std::max(s->smem, pic_particle_smem_bytes(mirror.dim, mirror.order, mirror.T));
     return PIC_OK;
 }
 
