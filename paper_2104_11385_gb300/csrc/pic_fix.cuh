@@ -250,8 +250,8 @@ struct TileBits {
 // NaN among others) is gathered in FP64
 __device__ __forceinline__ bool tile_exp_ok(int e) { return e == 0 || (e >= 128 && e <= 1900); }
 
-// The weakest field that is gathered in fixed point, as the high word of a double:
-// 2^-10 (linear) or 2^-8 of the component's largest magnitude in the tile.  Error
+// The weakest field that is gathered in fixed point, as a double's exponent: 2^-10
+// (linear) or 2^-8 of the component's largest magnitude in the tile.  Error
 // of the gather against exact arithmetic, relative to the strongest node it
 // interpolates from, random nodes (rms, largest):
 //                           linear 3D            cubic 3D
@@ -263,7 +263,7 @@ __device__ __forceinline__ bool tile_exp_ok(int e) { return e == 0 || (e >= 128 
 // of 2^-7 costs the 256^3 foil 30 % of its particle kernel there, 2^-10 1 %.
 template <int ORDER>
 __device__ __forceinline__ unsigned weak_limit(int emax) {
-    return (unsigned)(emax - (ORDER == 1 ? 10 : 8)) << 20;
+    return (unsigned)(emax - (ORDER == 1 ? 10 : 8));
 }
 
 // a double in units of 2^(emax - 1022 - FB), rounded to nearest; emax: biased

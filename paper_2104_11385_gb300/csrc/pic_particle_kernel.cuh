@@ -427,6 +427,46 @@ static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, doubl
     }
 }
 
+// Scans a staged tile: emax, the biased exponent of each component's largest
+// magnitude, and emin, that of the weakest two neighbours along x that are not both
+// zero (of the weakest single element where windows of mark_weak have single nodes
+// along x).  No window is weaker than that, so most tiles need no marks.  Elements
+// are taken in a row, 62 per warp and round, two per lane from a 16-byte load.
+template <int ORDER>
+__device__ __forceinline__ void scan_tile(const double* __restrict__ sEB, int stride, int vol, bool ec, int* emax, int* emin) {
+    const int lane = threadIdx.x & 31;
+    const bool one = ORDER == 1 && ec;
+    unsigned mx[6], mn[6];  // high words, the smallest less one (zero becomes the largest)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        mx[c] = 0u;
+        mn[c] = 0xFFFFFFFFu;
+    }
+    for (int i0 = 62 * (threadIdx.x >> 5); i0 < vol; i0 += 62 * (blockDim.x >> 5)) {
+        const int i = min(i0 + 2 * lane, vol - 2);  // (vol is even: rows have even lengths)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            const uint4 v = *reinterpret_cast<const uint4*>(sEB + c * stride + i);
+            const unsigned e = v.y & 0x7FFFFFFFu, o = v.w & 0x7FFFFFFFu, next = __shfl_down_sync(0xffffffffu, e, 1);
+            const bool single = one && ((c < 3 ? c == 0 : c != 3));  // half nodes along x
+            const unsigned both = max(e, o), across = lane == 31 ? both : max(o, next);
+            mx[c] = max(mx[c], both);
+            mn[c] = min(mn[c], min((single ? e : both) - 1u, (single ? o : across) - 1u));
+        }
+    }
+    unsigned hi = 0u, lo = 0u;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        const unsigned a = __reduce_max_sync(0xffffffffu, mx[c]), b = __reduce_min_sync(0xffffffffu, mn[c]);
+        hi = lane == c ? a : hi;
+        lo = lane == c ? b : lo;
+    }
+    if (lane < 6) {
+        atomicMax(emax + lane, (int)(hi >> 20));
+        atomicMin(emin + lane, lo == 0xFFFFFFFFu ? 0x7FFF : (int)((lo + 1u) >> 20));
+    }
+}
+
 // Marks where a component of a staged tile is gathered in FP64: one bit of bits + c
 // * words for each window of 2 x 2 x 2 nodes (a single node along the half-node
 // directions of the energy-conserving linear gather), numbered by the element i of
@@ -437,10 +477,11 @@ static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, doubl
 // one of them off the crossing, random noise marks hardly a window.  Elements are
 // taken in a row across row ends, where windows belong to no particle.  A lane
 // takes two windows from two 16-byte loads: shared loads are what this costs,
-// waiting behind the other CTA's reductions.  1 to 5 us per staged tile (16^3
-// plasma 40.7 -> 41.9 us per step, 128^3 foil 1402 -> 1415; one window per 4-byte
-// load 1420).  Without a pass of its own, from the loads that find the largest
-// magnitude, the windows waiting in registers: 1463 (spills).
+// waiting behind the other CTA's reductions, 1 to 5 us per staged tile, and only
+// the tiles where scan_tile leaves it open pay that (particle kernel per step
+// without the marks / marked always / where needed: 16^3 plasma 40.0 / 41.9 / 40.3
+// us, foil of 32 x 64 x 128 cells and 541 thousand particles 264 / 280 / 263, 128^3
+// foil 1402 / 1419 / 1407).
 __device__ __forceinline__ int mark_word(int i) { return ((i >> 6) << 1) | (i & 1); }
 __device__ __forceinline__ int mark_bit(int i) { return (i >> 1) & 31; }
 template <int ORDER, int DIM>
@@ -450,7 +491,7 @@ __device__ __forceinline__ bool mark_weak(unsigned* __restrict__ bits, int words
     const bool one = ORDER == 1 && ec;
     unsigned lim[6];
 #pragma unroll
-    for (int c = 0; c < 6; ++c) lim[c] = emax[c] == 0 ? 0u : weak_limit<ORDER>(emax[c]);
+    for (int c = 0; c < 6; ++c) lim[c] = emax[c] == 0 ? 0u : weak_limit<ORDER>(emax[c]) << 20;
     const int n = vol - 2 - SZ - (DIM == 3 ? SX : 0);  // last pair of windows that lie in the tile
     unsigned any = 0u;
     for (int w = 2 * (threadIdx.x >> 5); w < words; w += 2 * (blockDim.x >> 5)) {
@@ -1976,6 +2017,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
     __shared__ unsigned s_qhead[QMAXWARPS], s_qtail[QMAXWARPS];
     __shared__ unsigned long long s_cost, s_time;
     __shared__ int s_emax[6];  // fixed-point tile: biased exponent of each component's largest magnitude
+    __shared__ int s_emin[6];  // and of its weakest place (scan_tile)
     __shared__ int s_some;     // whether a cell is marked as too weak for it (mark_weak)
 
     const int nlists = sd->meta[0];
@@ -2111,7 +2153,10 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     cur.t = t;
                     tile_origin(S, t, cur.o);
                     if (threadIdx.x == 0) {
-                        for (int c = 0; c < 6; ++c) s_emax[c] = 0;
+                        for (int c = 0; c < 6; ++c) {
+                            s_emax[c] = 0;
+                            s_emin[c] = 0x7FFF;
+                        }
                         s_some = 0;
                         fence_proxy_async();
                         mbar_expect_tx(&bar, (uint32_t)(6 * P.eb_vol * sizeof(double)));
@@ -2144,27 +2189,23 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                     if constexpr (PREC != 2) {
                         // E/B tile to fixed point in place: the exponent of each
                         // component's largest magnitude, then the values in its units
-                        for (int c = 0; c < 6; ++c) {
-                            unsigned mx = 0u;
-#pragma unroll 4
-                            for (int i = threadIdx.x; i < P.eb_vol; i += blockDim.x)
-                                mx = max(mx, (unsigned)__double2hiint(sEBd[c * P.eb_stride + i]) & 0x7FFFFFFFu);
-                            mx = __reduce_max_sync(0xffffffffu, mx);
-                            if (lane == 0) atomicMax(&s_emax[c], (int)(mx >> 20));
-                        }
+                        scan_tile<ORDER>(sEBd, P.eb_stride, P.eb_vol, S.ec != 0, s_emax, s_emin);
                         __syncthreads();
-                        bool fx = true;
-                        for (int c = 0; c < 6; ++c) fx = fx && tile_exp_ok(s_emax[c]);
+                        bool fx = true, some = false;
+                        for (int c = 0; c < 6; ++c) {
+                            const int em = s_emax[c];
+                            fx = fx && tile_exp_ok(em);
+                            some = some || (em != 0 && s_emin[c] < (int)weak_limit<ORDER>(em));
+                        }
                         if (fx) {
-                            if (mark_weak<ORDER, DIM>(s_bits, P.bit_words, sEBd, P.eb_stride, P.eb_vol, S.ebs[0], S.ebs[1],
-                                                      s_emax, S.ec != 0))
+                            if (some && mark_weak<ORDER, DIM>(s_bits, P.bit_words, sEBd, P.eb_stride, P.eb_vol, S.ebs[0],
+                                                              S.ebs[1], s_emax, S.ec != 0))
                                 s_some = 1;
                         } else {  // every cell: Inf, NaN, or magnitudes outside the exponent range
                             for (int i = threadIdx.x; i < 6 * P.bit_words; i += blockDim.x) s_bits[i] = ~0u;
                             s_some = 1;
                         }
-                        __syncthreads();
-                        weak = s_some ? s_bits : nullptr;
+                        if (some) __syncthreads();  // (marked before it is converted)
                         if (fx) {
                             for (int c = 0; c < 6; ++c) {
                                 const int em = s_emax[c];
@@ -2176,6 +2217,7 @@ __global__ void __launch_bounds__(256, MINB) pic_particle_kernel(const SchedDev*
                             }
                         }
                         __syncthreads();
+                        weak = s_some ? s_bits : nullptr;
                     }
                     if constexpr (PREC == 2) {
                         // E/B tile to FP32 in place, in rounds of 8 elements per thread
