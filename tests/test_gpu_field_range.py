@@ -75,3 +75,70 @@ def test_fields_falling_along_z(dim, order, energy, binades):
             # a few dozen roundings of 2^-53 (oracle and kernel), no cancellation, and the
             # 9 (27) units of a fixed-point gather from a node that has 2^51 or more: 1.2e-14
             assert np.abs(g[k][gi] / r[k][ri] - 1.0).max() < 1e-13, k
+
+
+@pytest.mark.parametrize("dim,order,energy,tile,threads", [
+    (3, 1, False, 8, 256), (3, 1, True, 8, 256), (3, 2, False, 4, 128), (3, 2, True, 8, 32), (3, 3, False, 8, 256),
+    (3, 3, True, 4, 256), (2, 1, False, 16, 64), (2, 1, True, 16, 256), (2, 2, False, 32, 256), (2, 2, True, 16, 256),
+    (2, 3, False, 32, 96)])
+@pytest.mark.parametrize("corner", [(2, 3, 5), (5, 6, 9), (1, 2, 12)])
+def test_weak_patch(dim, order, energy, tile, threads, corner):
+    """nodes [corner, corner + 7) hold fields 2^-40 of those around them: particles that
+    interpolate from the patch alone see it to FP64's accuracy"""
+    wl = plasma(dim, order, lambda cell, n: np.ones(cell[0].size, bool))
+    if tile == 32:
+        wl["box"] = (32, 1, 32)
+    sp = wl["species"][0]
+    r = np.random.default_rng(5)
+    for a, k in enumerate("xyz"):
+        if dim == 3 or a != 1:
+            # cells corner + 2 and corner + 3: supports reach 2 nodes below and 3 above
+            sp[k] = (corner[a] + 2 + r.uniform(0, 2, sp[k].size)) * wl["dx"][a]
+    for k in ("ux", "uy", "uz"):
+        sp[k] = np.zeros_like(sp[k])
+    if energy:
+        wl["gather"] = "energy"
+    fields = workloads.random_fields(9, wl["ncell"], amp=0.2)
+    s = tuple(slice(c, c + 7) for c in corner)
+    patch = [slice(None)] * 3
+    patch[0], patch[2] = s[2], s[0]
+    if dim == 3:
+        patch[1] = s[1]
+    for c in range(3):
+        fields[c] = fields[c].copy()
+        fields[c].reshape(wl["ncell"][::-1])[tuple(patch)] *= 2.0 ** -40
+    fields[3:] = [np.zeros_like(f) for f in fields[3:]]
+    sim, ref = make_gpu(wl, fields), make_oracle(wl, fields)
+    sim.set_launch(tile=tile, threads=threads)
+    sim.step(1)
+    ref.step(1)
+    g, r = sim.particles(0), ref.particles(0)
+    gi, ri = np.argsort(g["id"]), np.argsort(r["id"])
+    for k in ("ux", "uy", "uz"):
+        want = r[k][ri]
+        assert 0.0 < np.abs(want).max() < 1e-10
+        # dozens of roundings of 2^-53 relative to the patch's fields
+        assert np.abs(g[k][gi] - want).max() < 1e-13 * np.abs(want).max(), k
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+@pytest.mark.parametrize("order,energy", [(1, False), (1, True), (2, False), (3, True)])
+def test_fields_falling_along_x_and_y(axis, order, energy):
+    wl = plasma(3, order, lambda cell, n: np.all([(c >= 4) & (c < m - 4) for c, m in zip(cell, n)], axis=0))
+    if energy:
+        wl["gather"] = "energy"
+    ncell = wl["ncell"]
+    shape = [1, 1, 1]
+    shape[2 - axis] = ncell[axis]
+    ramp = np.broadcast_to((0.2 * 8.0 ** -np.arange(ncell[axis])).reshape(shape), ncell[::-1]).reshape(-1).copy()
+    sp = wl["species"][0]
+    for k in ("ux", "uy", "uz"):
+        sp[k] = np.zeros_like(sp[k])
+    fields = [ramp] * 3 + [np.zeros_like(ramp)] * 3
+    sim, ref = make_gpu(wl, fields), make_oracle(wl, fields)
+    sim.step(1)
+    ref.step(1)
+    g, r = sim.particles(0), ref.particles(0)
+    gi, ri = np.argsort(g["id"]), np.argsort(r["id"])
+    for k in ("ux", "uy", "uz"):
+        assert np.abs(g[k][gi] / r[k][ri] - 1.0).max() < 1e-13, k  # as along z
