@@ -43,7 +43,7 @@ struct pic_sim {
     int split = 16;
     int ctas = 0;
     int minb = 1;
-    int prec = 0;  // 0 FP64, 1 float-float, 2 FP32 particle push
+    int prec = 0;  // 0 FP64, 1 float-float or better (run as FP64), 2 FP32 particle push
     int ppt = 1;   // particles per thread per loop iteration
     size_t smem = 0;
     int64_t tiles_cap[PIC_MAXSP] = {0, 0, 0, 0};  // sort arrays allocated for this many tiles
