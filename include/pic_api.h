@@ -367,7 +367,7 @@ pic_status pic_bin_particles(const pic_grid_desc* grid, const double* x, const d
  *                 value it is interpolated from, or, where all of those lie
  *                 below 2^-4 (linear shapes) or 2^-2 (others) of the
  *                 component's largest magnitude in the staged tile, within
- *                 2^-46; below 2^-10 (2^-8) of it FP64 takes over.  A current
+ *                 2^-46; below 2^-10 (2^-8) of it within 2^-51 again.  A current
  *                 contribution is within 2^-53 of itself and 2^-54 of the
  *                 charge that the particle carries in that direction;
  *                 2 float-float or better: runs the arithmetic of 1, which is

@@ -14,8 +14,8 @@
 //           component in the tile; FB = 62 for linear shapes, 60 for the
 //           others (headroom of the row sums).  A value down to 2^-9 (2^-7) of
 //           the largest keeps a double's 53 bits, a smaller one fewer: the tile's
-//           cells where a component is weak are marked when it is staged
-//           (weak_limit), and their particles gather it in FP64
+//           places where a component is weak are marked when it is staged
+//           (weak_limit), and their particles gather it by itself
 //   Amp     a floating-point factor: 64-bit mantissa, exponent, sign
 // Only the last step of each chain returns to IEEE doubles, by bit operations
 // and with one rounding: the six field values, and every current contribution.
@@ -258,7 +258,8 @@ __device__ __forceinline__ bool tile_exp_ok(int e) { return e == 0 || (e >= 128 
 //   nodes near the largest  1.5e-17, 1.0e-16     8.4e-18, 5.7e-17
 //   nodes at the limit      1.7e-15, 1.4e-14     1.4e-15, 7.5e-15
 //   FP64                    3.7e-17, 3.9e-16     3.7e-17, 3.5e-16
-// so a weak place keeps 46 bits or more, and FP64's where it is weaker still.  A
+// so a weak place keeps 46 bits or more, and all of them where it is weaker still:
+// there a component is gathered by itself, in units of its own nodes' largest.  A
 // laser on a foil has whole layers between 2^-7 and 2^-10 behind the skin: a limit
 // of 2^-7 costs the 256^3 foil 30 % of its particle kernel there, 2^-10 1 %.
 template <int ORDER>

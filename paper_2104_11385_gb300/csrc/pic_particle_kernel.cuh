@@ -385,8 +385,8 @@ __device__ __forceinline__ Six gather6_q(const long long* __restrict__ F, int st
     return r;
 }
 
-// Component c of the same in FP64 from the global arrays (which the kernel only
-// reads), out of line: for particles in cells where it is marked as weak.
+// Component c in FP64 from the global arrays (which the kernel only reads), out of
+// line: Inf, NaN, and magnitudes outside the fixed-point exponent range.
 template <int ORDER, int DIM>
 static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, double X, double Y, double Z, int ox, int oy,
                                                    int oz) {
@@ -425,6 +425,70 @@ static __device__ __noinline__ double gather1_fp64(const SimDev& S, int c, doubl
         }
         return v;
     }
+}
+
+// Component c in fixed point from the global arrays, in units of the largest
+// magnitude of the particle's own nodes, out of line: for particles where the
+// component is marked as weak against its tile's largest.  In FP64 it would hold
+// that pipe for 13 instructions of 16 clocks (linear 3D; cubic about 100) against
+// about 230 (1000) integer ones at a quarter of a clock.  The first steps of the 2D
+// cubic disk at 960^2 cells from zero fields, where noise fields span many
+// binades: 4.35 ms per step (in FP64 5.1; with the bits lost 3.4); all components of
+// a particle in one call: the same.  Rolled for long shapes, few registers: what a
+// call clobbers is spilled around it on the caller's fast path too.
+template <int ORDER, int DIM>
+static __device__ __noinline__ double gather1_weak(const SimDev& S, int c, double X, double Y, double Z, int ox, int oy,
+                                                   int oz) {
+    constexpr int FB = TileBits<ORDER>::FB, NY = DIM == 3 ? ORDER : 0;
+    const bool ec = S.ec != 0, isb = c >= 3;
+    const int a = isb ? c - 3 : c;
+    auto axis = [&](double x, int o, bool half) {
+        const CellQ q = cell_q(x);
+        const SupQ<ORDER> n = node_support<ORDER>(q, o), h = half_support<ORDER>(q, o, ec);
+        return axis_of<ORDER>(half ? h : n);
+    };
+    const AxisQ<ORDER> sx = axis(X, ox, (a == 0) != isb), sz = axis(Z, oz, (a == 2) != isb);
+    AxisQ<ORDER> sy = sx;
+    if (DIM == 3) sy = axis(Y, oy, (a == 1) != isb);
+    const double* const F = S.F[c] + pidx(S, ox + sx.s, DIM == 3 ? oy + sy.s : 0, oz + sz.s);
+    const int64_t px = S.pn[0], pxy = px * S.pn[1];
+    constexpr int U = ORDER == 1 ? 2 : 1;
+    unsigned m = 0u;
+#pragma unroll U
+    for (int k = 0; k <= ORDER; ++k)
+#pragma unroll U
+        for (int j = 0; j <= NY; ++j)
+#pragma unroll
+            for (int i = 0; i <= ORDER; ++i)
+                m = max(m, (unsigned)__double2hiint(F[k * pxy + j * px + i]) & 0x7FFFFFFFu);
+    const int em = (int)(m >> 20);
+    if (em < 128 || !tile_exp_ok(em)) return gather1_fp64<ORDER, DIM>(S, c, X, Y, Z, ox, oy, oz);
+    auto at = [&](int k, int j, int i) { return tile_fix<FB>(F[k * pxy + j * px + i], em); };
+    long long r;
+    if constexpr (ORDER == 1) {
+        auto row = [&](int k, int j) { return lerpq(at(k, j, 0), at(k, j, 1), sx.w[1]); };
+        if constexpr (DIM == 3)
+            r = lerpq(lerpq(row(0, 0), row(0, 1), sy.w[1]), lerpq(row(1, 0), row(1, 1), sy.w[1]), sz.w[1]);
+        else
+            r = lerpq(row(0, 0), row(1, 0), sz.w[1]);
+    } else {
+        AccQ vol;
+#pragma unroll 1
+        for (int k = 0; k <= ORDER; ++k) {
+            AccQ pl;
+#pragma unroll 1
+            for (int j = 0; j <= NY; ++j) {
+                AccQ line;
+#pragma unroll
+                for (int i = 0; i <= ORDER; ++i) line.mac(at(k, j, i), sx.w[i]);
+                if constexpr (DIM == 3) pl.mac(line.get(), sy.w[j]);
+                else vol.mac(line.get(), sz.w[k]);
+            }
+            if constexpr (DIM == 3) vol.mac(pl.get(), sz.w[k]);
+        }
+        r = vol.get();
+    }
+    return fix_double(r, em + 63 - FB);
 }
 
 // Scans a staged tile: emax, the biased exponent of each component's largest
@@ -467,7 +531,7 @@ __device__ __forceinline__ void scan_tile(const double* __restrict__ sEB, int st
     }
 }
 
-// Marks where a component of a staged tile is gathered in FP64: one bit of bits + c
+// Marks where a component of a staged tile is gathered by itself (gather1_weak): one bit of bits + c
 // * words for each window of 2 x 2 x 2 nodes (a single node along the half-node
 // directions of the energy-conserving linear gather), numbered by the element i of
 // its lower corner (mark_bit), set if it does not reach weak_limit and is not all
@@ -520,7 +584,7 @@ __device__ __forceinline__ bool mark_weak(unsigned* __restrict__ bits, int words
     }
     return any != 0u;
 }
-// the components (bits) that a particle gathers in FP64, from its supports and the marks
+// the components (bits) that a particle gathers by itself, from its supports and the marks
 template <int ORDER, int DIM>
 __device__ __forceinline__ unsigned weak_components(const unsigned* __restrict__ bits, int words, int SX, int SY,
                                                     const SupQ<ORDER>* nd, const AxisQ<ORDER>* hf) {
@@ -1429,7 +1493,7 @@ __device__ __forceinline__ PIn read_staged(const double* slot) {
 
 // Gather, Boris push, and deposit of one particle, FP64.  The gather and the
 // deposit are fixed-point; emax: biased exponents of the staged tile's components;
-// weak: its cells where a component is gathered in FP64, nullptr if there is none.
+// weak: marks where a component is gathered by itself, nullptr if there is none.
 template <class R, int DIM, int ORDER, class SV, class SPV>
 __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const SimDev& SG, const Tile& tl,
                                            const double* __restrict__ sEB, const unsigned* __restrict__ weak,
@@ -1470,7 +1534,7 @@ __device__ __forceinline__ void push_one_q(const SV& S, const SPV& sp, const Sim
             while (mask != 0u) {
                 const int c = __ffs((int)mask) - 1;
                 mask &= mask - 1u;
-                const double v = gather1_fp64<ORDER, DIM>(SG, c, x0[0], x0[1], x0[2], tl.o[0], tl.o[1], tl.o[2]);
+                const double v = gather1_weak<ORDER, DIM>(SG, c, x0[0], x0[1], x0[2], tl.o[0], tl.o[1], tl.o[2]);
 #pragma unroll
                 for (int k = 0; k < 6; ++k) f.v[k] = c == k ? v : f.v[k];
             }
