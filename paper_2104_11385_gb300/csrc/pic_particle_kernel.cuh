@@ -16,10 +16,10 @@
 // takes one warp instruction per SM every 16 clocks, and a particle's gather,
 // push and deposit are 165 FP64 instructions, 2.73 ms at 86 % of that pipe.
 // The gather (60 of them) and the deposit (36) run in 64-bit fixed point on the
-// integer pipes instead (pic_fix.cuh), the Boris push keeps 51: 1.35 ms, about
-// 2700 issued instructions per 32 particles, issue slots 44 % and FP64 pipe
-// 58 % busy (16 warps per SM by registers: latency-bound between the two).  Each thread brackets its particle
-// loop with clock64(); the deltas are warp-reduced, summed in shared memory and
+// integer pipes instead (pic_fix.cuh), the Boris push keeps 51: 1.40 ms, 2717
+// issued instructions per 32 particles, issue slots 43 % and FP64 pipe 56 % busy
+// (16 warps per SM by registers: latency-bound between the two).  Each thread
+// brackets its particle loop with clock64(); the deltas are warp-reduced, summed in shared memory and
 // added once per unit to the box's cost -- the device-clock cost of
 // arXiv 2104.11385 Sec. 2.2 (Fig. 2a); thread 0 adds the %globaltimer span
 // of the unit's particle loops, averaged over the warps, to the box's
