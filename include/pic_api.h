@@ -178,8 +178,8 @@ enum { PIC_SCHED_LISTS = 0, PIC_SCHED_QUEUE = 1 };
  *               The mean, because a unit that leaves warps idle is charged for
  *               the share it uses; the loops alone, because the tile staging
  *               before them takes about as long for every small box and would
- *               hide how their work differs.  It is a fixed cost per unit, and
- *               counted as one (14 us) where cuts into units are compared.
+ *               hide how their work differs.  It is a fixed cost per unit, about
+ *               14 us, which the least size of a unit takes care of.
  *   w_p, w_c    heuristic weights (Sec. 3.3 footnotes: 0.75/0.25 knapsack,
  *               0.02/0.98 SFC).
  *   cap_factor  knapsack cap on units per worker, times the average (1.5).

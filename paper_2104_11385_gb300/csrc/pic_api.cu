@@ -418,38 +418,6 @@ void map_units(const pic_sim* s, const pic_lb_params& p, const std::vector<pic::
     }
 }
 
-// Cuts the boxes into units and maps them.  Where that balances badly by measured
-// costs (E < 0.8: few units, and particles of unequal cost), finer cuts are tried
-// too, and the one whose heaviest worker ends first is taken, every unit counted
-// with the 14 us a step that it costs by itself.  Foil of 64 x 96 x 64 cells and 393
-// thousand particles after the pulse has hit it: particle kernel 573 -> 516 us.
-void cut_and_map(const pic_sim* s, const pic_lb_params& p, const std::vector<double>& costs, const std::vector<int64_t>& np,
-                 int64_t steps, int nw, std::vector<pic::Unit>& units, std::vector<double>& uc, std::vector<int32_t>& assign) {
-    const int64_t nb = s->h.nboxes;
-    const int split = p.split > 0 ? p.split : s->split;
-    int64_t least = pic::min_unit_particles(np.data(), nb, nw);
-    units = pic::make_units(costs.data(), np.data(), nb, nw, split, least, true);
-    map_units(s, p, units, nw, uc, assign);
-    if (p.cost == PIC_COST_HEURISTIC || p.policy == PIC_POLICY_BOX_ORDER || steps <= 0 ||
-        pic::lb_efficiency(uc.data(), assign.data(), (int64_t)uc.size(), nw) >= 0.8)
-        return;
-    const double unit_us = 14.0;  // in ns, or in clocks of a CTA's threads at 2 GHz
-    const double ov = (double)steps * unit_us * (p.cost == PIC_COST_KERNEL_TIME ? 1e3 : 2e3 * s->threads);
-    double best = pic::makespan(uc.data(), assign.data(), (int64_t)uc.size(), nw, ov);
-    while ((least /= 2) >= 256) {
-        std::vector<pic::Unit> u2 = pic::make_units(costs.data(), np.data(), nb, nw, split, least, true);
-        std::vector<double> c2;
-        std::vector<int32_t> a2;
-        map_units(s, p, u2, nw, c2, a2);
-        const double t = pic::makespan(c2.data(), a2.data(), (int64_t)c2.size(), nw, ov);
-        if (t >= best) continue;
-        best = t;
-        units.swap(u2);
-        uc.swap(c2);
-        assign.swap(a2);
-    }
-}
-
 pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_result* out) {
     std::vector<double> costs;
     std::vector<int64_t> np;
@@ -458,10 +426,12 @@ pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_re
     const int nw = n_workers_for(s, p);
     // E_old: the mapping in force, re-costed with the costs just measured
     const double e_old = plan_efficiency(s, costs);
-    std::vector<pic::Unit> units;
+    const int split = p.split > 0 ? p.split : s->split;
+    std::vector<pic::Unit> units =
+        pic::make_units(costs.data(), np.data(), nb, nw, split, pic::min_unit_particles(np.data(), nb, nw), true);
     std::vector<double> uc;
     std::vector<int32_t> assign;
-    cut_and_map(s, p, costs, np, s->cost_steps, nw, units, uc, assign);
+    map_units(s, p, units, nw, uc, assign);
     double e_new = pic::lb_efficiency(uc.data(), assign.data(), (int64_t)uc.size(), nw);
     bool adopted = pic::adopt(e_old, e_new, theta);
     if (adopted) {
@@ -470,8 +440,6 @@ pic_status rebalance(pic_sim* s, const pic_lb_params& p, double theta, pic_lb_re
     }
     s->last_costs = costs;
     s->last_np = np;
-    s->last_steps = s->cost_steps;
-    s->cost_steps = 0;
     CU(s, cudaMemsetAsync(s->h.cost_clock, 0, nb * sizeof(uint64_t), s->stream));
     CU(s, cudaMemsetAsync(s->h.cost_time, 0, nb * sizeof(uint64_t), s->stream));
     pic_lb_result r;
@@ -642,10 +610,13 @@ pic_status replan(pic_sim* s) {
     pic_lb_params p = s->lb_set ? s->lb : default_lb();
     if (p.mode == PIC_LB_NONE || s->last_costs.empty()) return initial_plan(s);
     const int nw = n_workers_for(s, p);
-    std::vector<pic::Unit> units;
+    const int split = p.split > 0 ? p.split : s->split;
+    std::vector<pic::Unit> units =
+        pic::make_units(s->last_costs.data(), s->last_np.data(), s->h.nboxes, nw, split,
+                        pic::min_unit_particles(s->last_np.data(), s->h.nboxes, nw), true);
     std::vector<double> uc;
     std::vector<int32_t> assign;
-    cut_and_map(s, p, s->last_costs, s->last_np, s->last_steps, nw, units, uc, assign);  // the simulation's own policy
+    map_units(s, p, units, nw, uc, assign);  // the simulation's own policy
     build_plan(s, units, assign, nw, p.sched, p.policy == PIC_POLICY_BOX_ORDER);
     return upload_plan(s);
 }
@@ -1102,7 +1073,6 @@ pic_status pic_step(pic_sim* s, int nsteps) {
         st.launches += s->kernels_per_step ? s->kernels_per_step : count_kernels(s);
         st.particle_launches += s->h.nsp > 0 ? 1 : 0;
         s->step_count++;
-        s->cost_steps++;
         const pic_lb_params& p = s->lb;
         if (s->lb_set && p.mode != PIC_LB_NONE && s->step_count % p.interval == 0) {
             if (p.mode == PIC_LB_DYNAMIC) {
@@ -1172,7 +1142,6 @@ pic_status pic_get_efficiency(pic_sim* s, int strategy, int reset_window, double
     if (reset_window) {
         CU(s, cudaMemsetAsync(s->h.cost_clock, 0, s->h.nboxes * sizeof(uint64_t), s->stream));
         CU(s, cudaMemsetAsync(s->h.cost_time, 0, s->h.nboxes * sizeof(uint64_t), s->stream));
-        s->cost_steps = 0;
         CU(s, cudaStreamSynchronize(s->stream));
     }
     return PIC_OK;

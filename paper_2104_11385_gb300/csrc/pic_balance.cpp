@@ -166,11 +166,4 @@ int64_t unit_share(int64_t nu, int ctas, int64_t np) {
     return std::max<int64_t>(1, std::min<int64_t>(ctas / nu, np / nu / 256));
 }
 
-double makespan(const double* costs, const int32_t* assign, int64_t nunits, int n_workers, double overhead) {
-    std::vector<double> load(n_workers, 0.0);
-    double mx = 0.0;
-    for (int64_t u = 0; u < nunits; ++u) mx = std::max(mx, load[assign[u]] += costs[u] + overhead);
-    return mx;
-}
-
 }  // namespace pic

@@ -32,7 +32,5 @@ std::vector<Unit> make_units(const double* costs, const int64_t* np, int64_t nbo
 int64_t min_unit_particles(const int64_t* np, int64_t nboxes, int n_workers);
 // CTAs that share each of nu uploaded units of np particles in all (1: none do)
 int64_t unit_share(int64_t nu, int ctas, int64_t np);
-// the heaviest worker's load when every unit costs `overhead` on top of its own
-double makespan(const double* costs, const int32_t* assign, int64_t nunits, int n_workers, double overhead);
 
 }  // namespace pic

@@ -489,7 +489,6 @@ pic_status pic_shard_finish(pic_sim* s, int advance) {
     if (advance) {
         SCU(s, pic_launch_finish(s->d, s->ds, PIC_SORT_NONE, s->stream));
         s->step_count++;
-        s->cost_steps++;
     }
     STRY(pic_sim_sync(s));
     return pic_sim_pull(s);

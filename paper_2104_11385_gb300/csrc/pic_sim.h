@@ -54,8 +54,6 @@ struct pic_sim {
     SimPlan plan;
     std::vector<double> last_costs;
     std::vector<int64_t> last_np;
-    int64_t cost_steps = 0;  // steps since the measured costs were last reset
-    int64_t last_steps = 0;  // steps that last_costs hold
     int64_t step_count = 0;
     std::vector<int32_t> box_ijk;
     // graph

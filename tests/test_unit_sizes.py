@@ -12,7 +12,6 @@ SHIM = r"""
 extern "C" {
 int64_t t_min(const int64_t* np, int64_t nb, int nw) { return pic::min_unit_particles(np, nb, nw); }
 int64_t t_share(int64_t nu, int ctas, int64_t np) { return pic::unit_share(nu, ctas, np); }
-double t_span(const double* c, const int32_t* a, int64_t n, int nw, double o) { return pic::makespan(c, a, n, nw, o); }
 }
 """
 
@@ -26,7 +25,6 @@ def lib(tmp_path_factory):
     subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-I", csrc, str(d / "shim.cpp"), "-o", str(so)])
     L = ctypes.CDLL(str(so))
     L.t_min.restype = L.t_share.restype = ctypes.c_int64
-    L.t_span.restype = ctypes.c_double
     return L
 
 
@@ -62,14 +60,6 @@ def test_few_boxes_leave_no_worker_idle(lib):
     """64 boxes, half of them empty, 4096 particles in the others, 304 workers"""
     counts = np.where(np.arange(64) % 2 == 0, 4096, 0)
     assert units(counts, least(lib, counts, 304)) >= 272
-
-
-def test_makespan(lib):
-    c = np.array([5.0, 1.0, 1.0, 3.0])
-    a = np.array([0, 1, 1, 2], np.int32)
-    f = lambda o: lib.t_span(c.ctypes.data_as(ctypes.c_void_p), a.ctypes.data_as(ctypes.c_void_p), ctypes.c_int64(4), 3,
-                             ctypes.c_double(o))
-    assert f(0.0) == 5.0 and f(1.0) == 6.0 and f(4.0) == 10.0
 
 
 @pytest.mark.parametrize("nu,ctas,np_,want", [(8, 152, 32768, 16), (8, 152, 400, 1), (8, 152, 0, 1), (76, 152, 10 ** 6, 2),
